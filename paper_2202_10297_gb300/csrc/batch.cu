@@ -115,7 +115,7 @@ __device__ void prod_reduce_tile(const adpar_batch_segment& sg, char* st, const 
     const T* x = static_cast<const T*>(sg.x);
     const int64_t lo = (int64_t)r * RT, hi = std::min<int64_t>(sg.len, lo + RT);
     range_prefetch_l2(x, lo, hi);
-    ProdStateQ ps = ProdStateQ::id();  // fixed-point products: no FP64 per element
+    ProdAcc ps = ProdAcc::id();  // fixed-point products: no FP64 per element
     constexpr int V = Vec16<T>::N;
     for (int64_t i = lo + threadIdx.x * V; i < hi; i += 256 * V) {
         if (i + V <= hi) {
@@ -126,7 +126,7 @@ __device__ void prod_reduce_tile(const adpar_batch_segment& sg, char* st, const 
             for (int64_t j = i; j < hi; ++j) ps.push(x[j], j);
         }
     }
-    ProdStateQ bs = block_reduce_256<ProdStateQ>(ps, prod_comb, s_warp);
+    ProdStateQ bs = block_reduce_256<ProdStateQ>(ps.state(), prod_comb, s_warp);
     ProdStateQ* partials = reinterpret_cast<ProdStateQ*>(st + L.partials);
     unsigned int* counter = reinterpret_cast<unsigned int*>(st + L.counter);
     if (threadIdx.x == 0) {
@@ -180,30 +180,41 @@ __device__ void prod_map_tile(const adpar_batch_segment& sg, char* st, const Sta
     double ym = 0.0;
     int64_t ye = 0;
     if (yb != 0.0) split_pow2(yb, ym, ye);
-    const double kq = f.m * ym;     // mantissa of p * ybar
-    const float qf = (float)kq;
-    for (int64_t i = lo + threadIdx.x; i < hi; i += 256) {
-        double c = 0.0;
-        if (yb != 0.0) {
-            if (f.nz == 0) {
-                if constexpr (sizeof(T) == 4) {  // FP32 output: FP32 arithmetic suffices
-                    float mf;
-                    int ef;
-                    split_pow2_f32m(static_cast<const float*>(sg.x)[i], mf, ef);
-                    xb[i] = scale_pow2f(qf * __frcp_rn(mf), f.e + ye - ef);
-                    continue;
-                } else {
-                    double mi;
-                    int64_t ei;
-                    split_pow2((double)x[i], mi, ei);
-                    c = scale_pow2(quot_mantissa(kq, mi), f.e + ye - ei);
-                }
-            } else if (f.nz == 1 && i == f.first) {
-                c = ldexp_clamped(f.m * ym, f.e + ye);
+    const double kq = f.m * ym;  // mantissa of p * ybar
+    if (f.nz == 0 && yb != 0.0) {
+        // every element: p / x_i * ybar, two 16-byte vectors in flight per thread
+        const int64_t e = f.e + ye;
+        const float qf = (float)kq;
+        const QuotF64 quot = QuotF64::make(kq, e);
+        auto one = [&](T v) -> T {
+            if constexpr (sizeof(T) == 4) return quot_f32(qf, e, v);
+            else return quot(v);
+        };
+        constexpr int V = Vec16<T>::N;
+        const int64_t whole = lo + (hi - lo) / V * V;
+        int64_t i = lo + threadIdx.x * V;
+        for (; i + 256 * V < whole; i += 512 * V) {
+            Vec16<T> u = ld_vec_stream(x + i), w = ld_vec_stream(x + i + 256 * V);
+#pragma unroll
+            for (int k = 0; k < V; ++k) {
+                u.v[k] = one(u.v[k]);
+                w.v[k] = one(w.v[k]);
             }
+            st_vec(xb + i, u);
+            st_vec(xb + i + 256 * V, w);
         }
-        xb[i] = (T)c;
+        if (i < whole) {
+            Vec16<T> u = ld_vec_stream(x + i);
+#pragma unroll
+            for (int k = 0; k < V; ++k) u.v[k] = one(u.v[k]);
+            st_vec(xb + i, u);
+        }
+        if (whole + threadIdx.x < hi) xb[whole + threadIdx.x] = one(x[whole + threadIdx.x]);
+        return;
     }
+    // a zero among the elements: its own adjoint (when it is the only one), 0 elsewhere
+    for (int64_t i = lo + threadIdx.x; i < hi; i += 256)
+        xb[i] = (f.nz == 1 && i == f.first && yb != 0.0) ? (T)ldexp_clamped(kq, f.e + ye) : T(0);
 }
 
 // linear-recurrence tile j of a segment: forward (adjoint false, left to

@@ -203,14 +203,14 @@ __global__ void __launch_bounds__(kRedBlock) reduce_arg_kernel(ReduceArgs A) {
 // The recompute multiplies mantissas in fixed point on the integer pipes
 // (no FP64 instruction per element for either dtype).
 template <class T>
-__global__ void __launch_bounds__(kRedBlock) reduce_prod_kernel(ReduceArgs A) {
+__global__ void __launch_bounds__(kRedBlock, 4) reduce_prod_kernel(ReduceArgs A) {
     using S = ProdStateQ;
     __shared__ S s_warp[kRedBlock / 32];
     const T* a = static_cast<const T*>(A.a);
     constexpr int V = Vec16<T>::N;
     const int64_t nvec = A.n / V;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    S st = S::id();
+    ProdAcc st = ProdAcc::id();
     constexpr int U = 4;  // vectors in flight per thread
     int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     for (; v + (U - 1) * stride < nvec; v += U * stride) {
@@ -232,7 +232,7 @@ __global__ void __launch_bounds__(kRedBlock) reduce_prod_kernel(ReduceArgs A) {
         st.push(a[i], i);
     }
     auto comb = [](const S& x, const S& y) { return S::comb(x, y); };
-    S bs = block_reduce(st, comb, s_warp);
+    S bs = block_reduce(st.state(), comb, s_warp);
     if (threadIdx.x == 0) static_cast<S*>(A.partials)[blockIdx.x] = bs;
     if (!last_block(A.hdr)) return;
     S totq = S::id();
@@ -276,7 +276,6 @@ __device__ __forceinline__ void prod_adjoint_body(const ReduceArgs& A, const Pro
     double ym = 0.0;
     int64_t ye = 0;
     if (yb != 0.0) split_pow2(yb, ym, ye);
-    const float qf = (float)(st.m * ym);  // the FP32 path's factor, in [0.25, 1]
     const double lg_p = log(fabs(st.m)) + (double)st.e * 0.69314718055994530942;
     const double lg_y = yb != 0.0 ? log(fabs(yb)) : -CUDART_INF;
     const int sgn_py = (st.m > 0 ? 1 : -1) * (yb > 0 ? 1 : (yb < 0 ? -1 : 0));
@@ -308,70 +307,50 @@ __device__ __forceinline__ void prod_adjoint_body(const ReduceArgs& A, const Pro
         }
         return;
     }
-    if constexpr (sizeof(T) == 4) {
-        // FP32, no zero: abar_i = p / a_i * ybar in FP32 arithmetic with the
-        // exponent kept apart (qf = the mantissa of p * ybar), 4 per thread
-        if (st.nz == 0 && yb != 0.0) {
-            const int64_t nv = A.n / 4;
-            const int64_t eb = st.e + ye;
-            auto one = [&](float x) {
-                float mf;
-                int ef;
-                split_pow2_f32m(x, mf, ef);
-                return scale_pow2f(qf * __frcp_rn(mf), eb - ef);
-            };
-            for (int64_t v = t0; v < nv; v += stride) {
-                const float4 x = __ldcs(reinterpret_cast<const float4*>(a) + v);
-                float4 o = make_float4(one(x.x), one(x.y), one(x.z), one(x.w));
+    const double kq = st.m * ym;  // the numerator's mantissa, in [0.25, 1)
+    if (st.nz == 0 && yb != 0.0) {
+        // no zero: abar_i = p / a_i * ybar, from the end (what the recompute
+        // read last is still in L2), four 16-byte vectors in flight per thread
+        const int64_t eb = st.e + ye;
+        const float qf = (float)kq;
+        const QuotF64 quot = QuotF64::make(kq, eb);
+        auto one = [&](T x) -> T {
+            if constexpr (sizeof(T) == 4) return quot_f32(qf, eb, x);
+            else return quot(x);
+        };
+        constexpr int V = Vec16<T>::N, U = 4;
+        const int64_t nv = A.n / V;
+        int64_t v = nv - 1 - t0;
+        for (; v - (U - 1) * stride >= 0; v -= U * stride) {
+            Vec16<T> x[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) x[u] = ld_vec_stream(a + (v - u * stride) * V);
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+#pragma unroll
+                for (int k = 0; k < V; ++k) x[u].v[k] = one(x[u].v[k]);
+                T* o = abar + (v - u * stride) * V;
                 if (A.accumulate) {
-                    const float4 p = reinterpret_cast<const float4*>(abar)[v];
-                    o.x += p.x; o.y += p.y; o.z += p.z; o.w += p.w;
+#pragma unroll
+                    for (int k = 0; k < V; ++k) x[u].v[k] += o[k];
                 }
-                __stcs(reinterpret_cast<float4*>(abar) + v, o);
+                st_vec(o, x[u]);
             }
-            const int64_t i = nv * 4 + t0;
-            if (i < A.n) abar[i] = A.accumulate ? abar[i] + one(a[i]) : one(a[i]);
-            return;
         }
-    }
-    const double kq = st.m * ym;  // the FP64 path's numerator mantissa, in [0.25, 1)
-    if constexpr (sizeof(T) == 8) {
-        // FP64, no zero: abar_i = p / a_i * ybar, two elements per 16-byte vector
-        if (st.nz == 0 && yb != 0.0) {
-            const int64_t nv = A.n / 2;
-            const int64_t eb = st.e + ye;
-            auto one = [&](double x) {
-                double mi;
-                int64_t ei;
-                split_pow2(x, mi, ei);
-                return scale_pow2(quot_mantissa(kq, mi), eb - ei);
-            };
-            for (int64_t v = t0; v < nv; v += stride) {
-                const double2 x = __ldcs(reinterpret_cast<const double2*>(a) + v);
-                double2 o = make_double2(one(x.x), one(x.y));
-                if (A.accumulate) {
-                    const double2 p = reinterpret_cast<const double2*>(abar)[v];
-                    o.x += p.x;
-                    o.y += p.y;
-                }
-                __stcs(reinterpret_cast<double2*>(abar) + v, o);
-            }
-            if (t0 == 0 && (A.n & 1)) {
-                const int64_t i = A.n - 1;
-                abar[i] = A.accumulate ? abar[i] + one(a[i]) : one(a[i]);
-            }
-            return;
+        for (; v >= 0; v -= stride) {
+            Vec16<T> x = ld_vec_stream(a + v * V);
+#pragma unroll
+            for (int k = 0; k < V; ++k) x.v[k] = A.accumulate ? abar[v * V + k] + one(x.v[k]) : one(x.v[k]);
+            st_vec(abar + v * V, x);
         }
+        const int64_t i = nv * V + t0;
+        if (i < A.n) abar[i] = A.accumulate ? abar[i] + one(a[i]) : one(a[i]);
+        return;
     }
     for (int64_t i = t0; i < A.n; i += stride) {
         double c = 0.0;
         if (yb != 0.0) {
-            if (st.nz == 0) {
-                double mi;
-                int64_t ei;
-                split_pow2((double)a[i], mi, ei);
-                c = scale_pow2(quot_mantissa(kq, mi), st.e + ye - ei);
-            } else if (st.nz == 1 && i == st.first) {
+            if (st.nz == 1 && i == st.first) {
                 c = ldexp_clamped(st.m * ym, st.e + ye);
             }
         }
@@ -380,7 +359,7 @@ __device__ __forceinline__ void prod_adjoint_body(const ReduceArgs& A, const Pro
 }
 
 template <class T>
-__global__ void __launch_bounds__(kRedBlock) prod_adjoint_kernel(ReduceArgs A) {
+__global__ void __launch_bounds__(kRedBlock, 4) prod_adjoint_kernel(ReduceArgs A) {
     const ProdState st = *static_cast<const ProdState*>(A.final_state);
     prod_adjoint_body<T>(A, st, blockIdx.x * (int64_t)blockDim.x + threadIdx.x, (int64_t)gridDim.x * blockDim.x);
 }
@@ -396,6 +375,9 @@ size_t state_bytes(int op, int dtype) {
     }
     return 0;
 }
+
+// resident blocks of the * kernels: 4 of 256 threads on each of 152 SMs
+constexpr int kProdGrid = 4 * 152;
 
 int grid_for(int64_t n, int dtype) {
     const int64_t per_block = (int64_t)kRedBlock * (dtype == ADPAR_F64 ? 2 : 4) * 8;
@@ -417,10 +399,12 @@ int run_reduce(ReduceArgs A, int op, cudaStream_t s) {
         reduce_arg_kernel<T, true><<<grid, kRedBlock, 0, s>>>(A);
         break;
     case ADPAR_OP_MUL: {
-        reduce_prod_kernel<T><<<grid, kRedBlock, 0, s>>>(A);
+        // one 16-byte vector per thread, up to a whole wave of resident blocks
+        const int64_t per = (int64_t)kRedBlock * (16 / sizeof(T));
+        const int gp = (int)std::max<int64_t>(1, std::min<int64_t>((A.n + per - 1) / per, kProdGrid));
+        reduce_prod_kernel<T><<<gp, kRedBlock, 0, s>>>(A);
         if (A.primal_only) break;
-        const int g2 = (int)std::max<int64_t>(1, std::min<int64_t>((A.n + 1023) / 1024, 4 * 152));
-        prod_adjoint_kernel<T><<<g2, kRedBlock, 0, s>>>(A);
+        prod_adjoint_kernel<T><<<gp, kRedBlock, 0, s>>>(A);
         break;
     }
     default:
