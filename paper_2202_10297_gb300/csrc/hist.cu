@@ -23,6 +23,7 @@
 #include <math_constants.h>
 
 #include "common.cuh"
+#include "hist_logprod.cuh"
 #include "prod.cuh"
 #include "scan_ops.cuh"
 
@@ -77,26 +78,17 @@ struct HistArgs {
     long long* pe;            // [m] * : its exponent
     unsigned int* pz;         // [m] * : zero count
     long long* pf;            // [m] * : lowest zero index
-    struct BinQ* binq;        // [m] * with FP32 values: per-bin factor of the adjoint
-    int q62;                  // * with FP32 values: pm holds the fixed-point mantissa
+    // * over FP32 values by logarithm sums (hist_logprod.cuh): pz, pf and
+    ulonglong2* acc;  // [m] the bins' words
+    ulonglong2* tab;  // [kLogTab]
+    BinQ* binq;       // [m] factors of the adjoint
     // * : per-block partial states of the shared-memory bins [0, hw), merged
     // by hist_prod_merge_kernel ([blocks][hw] each)
     int64_t hw;
-    unsigned long long* part_m;
+    double* part_m;
     long long* part_e;
     long long* part_f;
     unsigned* part_z;
-};
-
-// Per-bin factor of the * adjoint for FP32 values (value domain): (qm, qe)
-// with P_nz * hsbar_b = qm * 2^qe, qm an FP32 mantissa (0.5 <= |qm| < 1),
-// and `sel`: -1 = the bin has no zero (every element gets P_nz/v_i * hsbar),
-// an index = the bin's only zero (that element gets P_nz * hsbar), -2 =
-// nothing (two or more zeros, or hsbar_b = 0).
-struct alignas(16) BinQ {
-    float qm;
-    int qe;
-    long long sel;
 };
 
 __global__ void hist_init_kernel(HistArgs A, unsigned long long key_empty) {
@@ -106,10 +98,9 @@ __global__ void hist_init_kernel(HistArgs A, unsigned long long key_empty) {
     for (int64_t b = t0; b < A.m; b += stride) {
         if (A.key) A.key[b] = key_empty;
         if (A.idx) A.idx[b] = 0xffffffffffffffffull;
-        if (A.pm) {  // the neutral product: fixed point 2^62 * 2^-62, or 0.5 * 2^1
-            if (A.q62) reinterpret_cast<unsigned long long*>(A.pm)[b] = 1ull << 62;
-            else A.pm[b] = 0.5;
-            A.pe[b] = A.q62 ? 0 : 1;
+        if (A.pm) {  // the neutral product, 0.5 * 2^1
+            A.pm[b] = 0.5;
+            A.pe[b] = 1;
             A.pz[b] = 0u;
             A.pf[b] = INT64_MAX;
         }
@@ -304,34 +295,22 @@ __device__ __forceinline__ void mul_into(double* pm, long long* pe, double mi, l
     if (shift) atomicAdd(reinterpret_cast<unsigned long long*>(pe), (unsigned long long)shift);
 }
 
-// global CAS: *pM = *pM * mv (fixed point); the exponent gets ev + the increment
-__device__ __forceinline__ void q62_mul24_into(unsigned long long* pM, long long* pE, unsigned mv, int ev) {
-    unsigned long long old = *reinterpret_cast<volatile unsigned long long*>(pM), assumed, nb;
-    int de;
-    do {
-        assumed = old;
-        nb = q62_mul24(assumed, mv, de);
-        old = atomicCAS(pM, assumed, nb);
-    } while (old != assumed);
-    atomicAdd(reinterpret_cast<unsigned long long*>(pE), (unsigned long long)(long long)(ev + de));
-}
-
-// A bin's recomputed state, for either representation.
-template <class T>
+// A bin's recomputed state.
 __device__ __forceinline__ void read_bin(const HistArgs& A, int64_t b, double& mm, int64_t& e, unsigned& nz) {
-    const unsigned z = A.pz[b];
-    if constexpr (sizeof(T) == 4) {
-        nz = z & 0x7fffffffu;
-        q62_to_pow2(reinterpret_cast<const unsigned long long*>(A.pm)[b], A.pe[b], z >> 31, mm, e);
-    } else {
-        nz = z;
-        int64_t ee;
-        split_pow2(A.pm[b], mm, ee);
-        e = A.pe[b] + ee;
+    nz = A.pz[b];
+    if (A.acc) {  // hist_logprod_bins_kernel left (mantissa, exponent) there
+        const ulonglong2 w = A.acc[b];
+        mm = __longlong_as_double((long long)w.x);
+        e = (int64_t)w.y;
+        return;
     }
+    int64_t ee;
+    split_pow2(A.pm[b], mm, ee);
+    e = A.pe[b] + ee;
 }
 
-// Bin tiers of the * recompute:
+// Bin tiers of the * recompute over FP64 values (and FP32 arrays of 2^32
+// elements and more):
 //   [0, H)       warp-private copies: lanes of a warp that hit the same bin
 //                are serialised into rounds (__match_any_sync picks one
 //                leader per bin per round), so every update is a plain
@@ -339,18 +318,15 @@ __device__ __forceinline__ void read_bin(const HistArgs& A, int64_t b, double& m
 //   [H, H + H2)  one block-shared copy updated with shared-memory CAS;
 //   the rest     global CAS (L2).
 // Rank-ordered skewed data (Zipf) keeps its hot bins in the first tiers.
-// FP32 values use the fixed-point state above in every tier; FP64 values
-// an FP64 mantissa in [0.5, 1) and an integer exponent.
 constexpr int kProdWarpBins = 256;
 constexpr int kProdBlockBins = 2048;
 constexpr int kProdBlock = 256;
 constexpr int kProdMaxGrid = 1024;  // rows of the partial-state arrays
 
-// One warp-private bin: mantissa (fixed point, or FP64 bits), exponent and
-// zero count (with the sign parity in bit 31 for fixed point), read and
+// One warp-private bin: FP64 mantissa, exponent and zero count, read and
 // written as one 16-byte word.
 struct alignas(16) WBin {
-    unsigned long long M;
+    double M;
     int E;
     unsigned Z;
 };
@@ -358,46 +334,29 @@ struct alignas(16) WBin {
 template <class T, class I>
 __global__ void __launch_bounds__(kProdBlock, 4) hist_prod_kernel(HistArgs A) {
     extern __shared__ unsigned char smem_raw[];
-    constexpr bool kQ = sizeof(T) == 4;
     constexpr int NW = kProdBlock / 32;
     const int H = (int)std::min<int64_t>(A.m, kProdWarpBins);
     WBin* wb = reinterpret_cast<WBin*>(smem_raw);              // [NW][H]
     long long* wf = reinterpret_cast<long long*>(wb + NW * H);  // [NW][H] lowest zero index
     const int H2 = (int)std::max<int64_t>(0, std::min<int64_t>(A.m - H, kProdBlockBins));
-    unsigned long long* bm = reinterpret_cast<unsigned long long*>(wf + NW * H);  // [H2] block-shared tier
+    double* bm = reinterpret_cast<double*>(wf + NW * H);  // [H2] block-shared tier
     long long* be = reinterpret_cast<long long*>(bm + H2);
     long long* bf = be + H2;
     unsigned int* bz = reinterpret_cast<unsigned int*>(bf + H2);
-    const unsigned long long one = kQ ? kQ62One : (unsigned long long)__double_as_longlong(0.5);
-    const int e_one = kQ ? 0 : 1;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int q = threadIdx.x; q < NW * H; q += blockDim.x) {
-        wb[q] = WBin{one, e_one, 0u};
+        wb[q] = WBin{0.5, 1, 0u};
         wf[q] = INT64_MAX;
     }
     for (int q = threadIdx.x; q < H2; q += blockDim.x) {
-        bm[q] = one;
-        be[q] = e_one;
+        bm[q] = 0.5;
+        be[q] = 1;
         bf[q] = INT64_MAX;
         bz[q] = 0u;
     }
     __syncthreads();
     WBin* myb = wb + warp * H;
     long long* myf = wf + warp * H;
-    unsigned long long* gM = reinterpret_cast<unsigned long long*>(A.pm);
-    // FP32 values: each lane keeps the nonzero factors of bins [0, kHot) in
-    // registers (the hottest bins of rank-ordered skewed data), so they take
-    // no part in the warp's serialised rounds; merged once at the end
-    constexpr int kHot = kQ ? 8 : 0;
-    const int hot = (int)std::min<int64_t>(A.m, kHot);
-    unsigned long long cM[kHot > 0 ? kHot : 1];
-    int cE[kHot > 0 ? kHot : 1];
-    unsigned cS = 0;  // sign parities, bit k for bin k
-#pragma unroll
-    for (int k = 0; k < kHot; ++k) {
-        cM[k] = kQ62One;
-        cE[k] = 0;
-    }
     const I* inds = static_cast<const I*>(A.inds);
     const T* vals = static_cast<const T*>(A.vals);
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -405,59 +364,33 @@ __global__ void __launch_bounds__(kProdBlock, 4) hist_prod_kernel(HistArgs A) {
     for (int64_t it = 0; it < nround; ++it) {
         const int64_t i = it * stride + blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
         int64_t b = -1;
-        T v = T(0);
+        double v = 0.0;
         if (i < A.n) {
             b = ld_index(inds, i);
-            v = __ldcs(vals + i);
+            v = (double)__ldcs(vals + i);
         }
-        const bool zero = v == T(0);
-        // the element's factor: fixed point (sg, mv, ev) or FP64 (mi, ei)
-        unsigned sg = 0, mv = 0;
-        int ev = 0;
+        const bool zero = v == 0.0;
         double mi = 0.5;
         int64_t ei = 1;
         const bool in = b >= 0 && b < A.m;
-        if (in && !zero) {
-            if constexpr (kQ) split_f32_int(v, sg, mv, ev);
-            else split_pow2(v, mi, ei);
-        }
+        if (in && !zero) split_pow2(v, mi, ei);
         if (in && b >= H && b < H + H2) {  // warm bins: block-shared, shared-memory CAS
             const int q = (int)(b - H);
             if (zero) {
                 atomicAdd(bz + q, 1u);
                 atomicMin(bf + q, (long long)i);
-            } else if constexpr (kQ) {
-                q62_mul24_into(bm + q, be + q, mv, ev);
-                if (sg) atomicXor(bz + q, 0x80000000u);
             } else {
-                mul_into(reinterpret_cast<double*>(bm + q), be + q, mi, ei);
+                mul_into(bm + q, be + q, mi, ei);
             }
         } else if (in && b >= H + H2) {  // cold bins: global atomics
             if (zero) {
                 atomicAdd(A.pz + b, 1u);
                 atomicMin(A.pf + b, (long long)i);
-            } else if constexpr (kQ) {
-                q62_mul24_into(gM + b, A.pe + b, mv, ev);
-                if (sg) atomicXor(A.pz + b, 0x80000000u);
             } else {
                 mul_into(A.pm + b, A.pe + b, mi, ei);
             }
         }
         bool pending = in && b < H;
-        if constexpr (kHot > 0) {
-            if (pending && !zero && b < hot) {
-#pragma unroll
-                for (int k = 0; k < kHot; ++k) {
-                    if (b == k) {
-                        int de;
-                        cM[k] = q62_mul24(cM[k], mv, de);
-                        cE[k] += ev + de;
-                        cS ^= sg << k;
-                    }
-                }
-                pending = false;
-            }
-        }
         const unsigned key = pending ? (unsigned)b : (0x80000000u | (unsigned)lane);
         while (__any_sync(0xffffffffu, pending)) {
             const unsigned grp = __match_any_sync(0xffffffffu, pending ? key : (0x80000000u | (unsigned)lane));
@@ -467,16 +400,10 @@ __global__ void __launch_bounds__(kProdBlock, 4) hist_prod_kernel(HistArgs A) {
                 if (zero) {
                     x.Z += 1;
                     if (i < myf[b]) myf[b] = i;
-                } else if constexpr (kQ) {
-                    int de;
-                    x.M = q62_mul24(x.M, mv, de);
-                    x.E += ev + de;
-                    x.Z ^= sg << 31;
                 } else {
-                    double mm = __longlong_as_double((long long)x.M) * mi;
+                    x.M *= mi;
                     int64_t e2 = 0;
-                    renorm(mm, e2);
-                    x.M = (unsigned long long)__double_as_longlong(mm);
+                    renorm(x.M, e2);
                     x.E += (int)(ei + e2);
                 }
                 myb[b] = x;
@@ -485,69 +412,26 @@ __global__ void __launch_bounds__(kProdBlock, 4) hist_prod_kernel(HistArgs A) {
             __syncwarp();
         }
     }
-    // the lanes' register bins: a shuffle tree per bin, then lane 0 folds
-    // the warp's product into its shared-memory copy
-    if constexpr (kHot > 0) {
-#pragma unroll
-        for (int k = 0; k < kHot; ++k) {
-            unsigned long long M = cM[k];
-            long long E = cE[k];
-            unsigned sgn = (cS >> k) & 1u;
-#pragma unroll
-            for (int off = 16; off; off >>= 1) {
-                const unsigned long long M2 = __shfl_xor_sync(0xffffffffu, M, off);
-                const long long E2 = __shfl_xor_sync(0xffffffffu, E, off);
-                int de;
-                M = q62_mul(M, M2, de);
-                E += E2 + de - 62;
-                sgn ^= __shfl_xor_sync(0xffffffffu, sgn, off);
-            }
-            if (lane == 0 && k < hot) {
-                WBin x = myb[k];
-                int de;
-                x.M = q62_mul(x.M, M, de);
-                x.E += (int)(E + de - 62);
-                x.Z ^= sgn << 31;
-                myb[k] = x;
-            }
-        }
-    }
     __syncthreads();
     // this block's state of the shared-memory bins goes to its partial row
     // (no global atomics); hist_prod_merge_kernel combines the rows
     const int64_t row = (int64_t)blockIdx.x * A.hw;
     for (int q = threadIdx.x; q < H; q += blockDim.x) {
-        unsigned nz = 0, sign = 0;
+        unsigned nz = 0;
         long long first = INT64_MAX;
-        unsigned long long M;
-        long long E;
-        if constexpr (kQ) {
-            M = kQ62One;
-            E = 0;
-        } else {
-            M = (unsigned long long)__double_as_longlong(0.5);
-            E = 1;
-        }
+        double M = 0.5;
+        int64_t E = 1;
         for (int w = 0; w < NW; ++w) {
             const WBin x = wb[w * H + q];
-            nz += x.Z & 0x7fffffffu;
-            sign ^= x.Z >> 31;
+            nz += x.Z;
             first = std::min(first, wf[w * H + q]);
-            if constexpr (kQ) {
-                int de;
-                M = q62_mul(M, x.M, de);
-                E += x.E + de - 62;
-            } else {
-                double mm = __longlong_as_double((long long)M) * __longlong_as_double((long long)x.M);
-                int64_t e2 = 0;
-                renorm(mm, e2);
-                M = (unsigned long long)__double_as_longlong(mm);
-                E += x.E + e2;
-            }
+            M *= x.M;
+            E += x.E;
+            renorm(M, E);
         }
         A.part_m[row + q] = M;
         A.part_e[row + q] = E;
-        A.part_z[row + q] = nz | (sign << 31);
+        A.part_z[row + q] = nz;
         A.part_f[row + q] = first;
     }
     for (int q = threadIdx.x; q < H2; q += blockDim.x) {
@@ -561,50 +445,34 @@ __global__ void __launch_bounds__(kProdBlock, 4) hist_prod_kernel(HistArgs A) {
 // Combines the per-block partial states of the shared-memory bins: one
 // warp per bin, lanes take every 32nd block row, then a shuffle tree.  It is
 // the only writer of these bins' global state.
-template <class T>
 __global__ void hist_prod_merge_kernel(HistArgs A, int rows) {
-    constexpr bool kQ = sizeof(T) == 4;
     const int lane = threadIdx.x & 31;
     const int64_t b = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     if (b >= A.hw) return;
-    unsigned long long M = kQ ? kQ62One : (unsigned long long)__double_as_longlong(0.5);
-    long long E = kQ ? 0 : 1;
-    unsigned nz = 0, sign = 0;
+    double M = 0.5;
+    int64_t E = 1;
+    unsigned nz = 0;
     long long first = INT64_MAX;
-    auto comb = [](unsigned long long& M1, long long& E1, unsigned long long M2, long long E2) {
-        if constexpr (kQ) {
-            int de;
-            M1 = q62_mul(M1, M2, de);
-            E1 += E2 + de - 62;
-        } else {
-            double mm = __longlong_as_double((long long)M1) * __longlong_as_double((long long)M2);
-            int64_t e2 = 0;
-            renorm(mm, e2);
-            M1 = (unsigned long long)__double_as_longlong(mm);
-            E1 += E2 + e2;
-        }
-    };
     for (int r = lane; r < rows; r += 32) {
         const int64_t k = (int64_t)r * A.hw + b;
-        comb(M, E, A.part_m[k], A.part_e[k]);
-        const unsigned z = A.part_z[k];
-        nz += z & 0x7fffffffu;
-        sign ^= z >> 31;
+        M *= A.part_m[k];
+        E += A.part_e[k];
+        renorm(M, E);
+        nz += A.part_z[k];
         first = std::min(first, A.part_f[k]);
     }
 #pragma unroll
     for (int off = 16; off; off >>= 1) {
-        const unsigned long long M2 = __shfl_xor_sync(0xffffffffu, M, off);
-        const long long E2 = __shfl_xor_sync(0xffffffffu, E, off);
-        comb(M, E, M2, E2);
+        M *= __shfl_xor_sync(0xffffffffu, M, off);
+        E += __shfl_xor_sync(0xffffffffu, (long long)E, off);
+        renorm(M, E);
         nz += __shfl_xor_sync(0xffffffffu, nz, off);
-        sign ^= __shfl_xor_sync(0xffffffffu, sign, off);
         first = std::min(first, (long long)__shfl_xor_sync(0xffffffffu, first, off));
     }
     if (lane == 0) {
-        A.pm[b] = __longlong_as_double((long long)M);  // the bits, in either representation
+        A.pm[b] = M;
         A.pe[b] = E;
-        A.pz[b] = kQ ? (nz | (sign << 31)) : nz;
+        A.pz[b] = nz;
         A.pf[b] = first;
     }
 }
@@ -617,7 +485,7 @@ __global__ void hist_prod_bins_kernel(HistArgs A) {
         double mm;
         int64_t e;
         unsigned nz;
-        read_bin<T>(A, b, mm, e, nz);
+        read_bin(A, b, mm, e, nz);
         if (A.hs_out) static_cast<T*>(A.hs_out)[b] = nz ? T(0) : (T)ldexp_clamped(mm, e);
         if (A.bin_aux) {
             adpar_prod_aux x;
@@ -651,8 +519,8 @@ __global__ void __launch_bounds__(kHistBlock) hist_prod_vjp_kernel(HistArgs A) {
             double mm;
             int64_t e;
             unsigned nz;
-            read_bin<T>(A, b, mm, e, nz);
-            if (yb != 0.0 && (nz == 0 || (nz == 1 && A.pf[b] == i))) {
+            read_bin(A, b, mm, e, nz);
+            if (yb != 0.0 && (nz == 0 || (nz == 1 && vals[i] == T(0)))) {  // the bin's only zero
                 double ym;
                 int64_t ye;
                 split_pow2(yb, ym, ye);
@@ -689,91 +557,35 @@ __global__ void __launch_bounds__(kHistBlock) hist_prod_vjp_kernel(HistArgs A) {
     }
 }
 
-// per-bin factors of the FP32 value-domain adjoint (see BinQ)
-template <class T>
-__global__ void hist_prod_binq_kernel(HistArgs A) {
-    const T* hsbar = static_cast<const T*>(A.hsbar);
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; b < A.m; b += stride) {
-        BinQ q;
-        q.qm = 0.0f;
-        q.qe = 0;
-        q.sel = -2;
-        const double yb = (double)hsbar[b];
-        double mm;
-        int64_t ee;
-        unsigned nz;
-        read_bin<T>(A, b, mm, ee, nz);
-        if (yb != 0.0 && nz <= 1) {
-            double ym, m2;
-            int64_t ye, e2;
-            split_pow2(yb, ym, ye);
-            split_pow2(mm * ym, m2, e2);  // in [0.25, 1): one more split
-            float qf = (float)m2;        // rounding may reach 1.0
-            int64_t e = ee + ye + e2;
-            if (fabsf(qf) >= 1.0f) {
-                qf *= 0.5f;
-                e += 1;
-            }
-            q.qm = qf;
-            q.qe = (int)(e > (1 << 30) ? (1 << 30) : (e < -(1 << 30) ? -(1 << 30) : e));
-            q.sel = nz == 0 ? -1 : A.pf[b];
-        }
-        A.binq[b] = q;
-    }
-}
-
-// per element, FP32 values in the value domain: the three cases of
-// Sec. 5.1.1 from the bin's factor, in FP32 arithmetic with the exponent
-// kept apart (qm / m_v, then 2^(qe - e_v) applied to the exponent field)
-template <class I>
-__global__ void __launch_bounds__(kHistBlock) hist_prod_vjp_f32_kernel(HistArgs A) {
-    const I* inds = static_cast<const I*>(A.inds);
-    const float* vals = static_cast<const float*>(A.vals);
-    float* vb = static_cast<float*>(A.valsbar);
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < A.n; i += stride) {
-        const int64_t b = ld_index(inds, i);
-        const bool in = b >= 0 && b < A.m;
-        float c = 0.0f;
-        if (in) {
-            const BinQ q = A.binq[b];
-            if (q.sel == -1) {
-                float mv;
-                int ev;
-                split_pow2_f32m(__ldcs(vals + i), mv, ev);
-                c = scale_pow2f(q.qm * __frcp_rn(mv), (int64_t)q.qe - ev);
-            } else if (q.sel == i) {
-                c = scale_pow2f(q.qm, (int64_t)q.qe);
-            }
-        }
-        if (A.accumulate) {
-            if (in) vb[i] += c;
-        } else {
-            vb[i] = c;
-        }
-    }
-}
-
 // ------------------------------------------------------------ host side
+// FP32 * by logarithm sums: within the words' range (every realistic call)
+bool use_logprod(int op, int dtype, int64_t n, int64_t m) {
+    return op == ADPAR_OP_MUL && dtype == ADPAR_F32 && n < (int64_t(1) << 32) && m < (int64_t(1) << 31);
+}
+
 struct HistLayout {
-    size_t off_key, off_idx, off_pm, off_pe, off_pz, off_pf, off_binq, off_part_m, off_part_e, off_part_f,
-        off_part_z, total;
+    size_t off_key, off_idx, off_pm, off_pe, off_pz, off_pf, off_acc, off_tab, off_binq, off_part_m, off_part_e,
+        off_part_f, off_part_z, total;
 };
 
-HistLayout hist_layout(int op, int dtype, int64_t m) {
+HistLayout hist_layout(int op, int dtype, int64_t n, int64_t m) {
     HistLayout L{};
     size_t o = sizeof(WsHeader);
     const size_t mm = (size_t)std::max<int64_t>(m, 1);
     if (op == ADPAR_OP_MIN || op == ADPAR_OP_MAX) {
         L.off_key = o; o = round_up(o + mm * 8, 256);
         if (dtype == ADPAR_F64) { L.off_idx = o; o = round_up(o + mm * 8, 256); }
+    } else if (use_logprod(op, dtype, n, m)) {
+        L.off_tab = o; o = round_up(o + kLogTab * 16, 256);
+        L.off_acc = o; o = round_up(o + mm * 16, 256);
+        L.off_pf = o; o = round_up(o + mm * 8, 256);
+        L.off_pz = o; o = round_up(o + mm * 4, 256);
+        L.off_binq = o; o = round_up(o + mm * sizeof(BinQ), 256);
     } else if (op == ADPAR_OP_MUL) {
         L.off_pm = o; o = round_up(o + mm * 8, 256);
         L.off_pe = o; o = round_up(o + mm * 8, 256);
         L.off_pf = o; o = round_up(o + mm * 8, 256);
         L.off_pz = o; o = round_up(o + mm * 4, 256);
-        if (dtype == ADPAR_F32) { L.off_binq = o; o = round_up(o + mm * sizeof(BinQ), 256); }
         const size_t hw = (size_t)std::min<int64_t>(m, kProdWarpBins + kProdBlockBins);
         const size_t np = hw * (size_t)kProdMaxGrid;
         L.off_part_m = o; o = round_up(o + np * 8, 256);
@@ -798,7 +610,7 @@ int run_hist(HistArgs A, cudaStream_t s) {
     const int gridN = (int)std::max<int64_t>(1, std::min<int64_t>((A.n + kHistBlock - 1) / kHistBlock, (int64_t)sms * 4));
     const int gridM = (int)std::max<int64_t>(1, std::min<int64_t>((A.m + 255) / 256, (int64_t)sms * 8));
     const int op = A.op;
-    if (op != ADPAR_OP_ADD) {
+    if (op != ADPAR_OP_ADD && !A.acc) {
         const unsigned long long empty = op == ADPAR_OP_MAX ? 0ull : 0xffffffffffffffffull;
         hist_init_kernel<<<gridM, 256, 0, s>>>(A, empty);
     }
@@ -831,6 +643,35 @@ int run_hist(HistArgs A, cudaStream_t s) {
         break;
     }
     case ADPAR_OP_MUL: {
+        if constexpr (sizeof(T) == 4) {
+            if (A.acc) {
+                LogProdArgs G{A.n, A.m, static_cast<const float*>(A.vals), A.inds, A.acc, A.pz,
+                              A.bin_aux ? A.pf : nullptr, A.tab};
+                const int gi = (int)std::max<int64_t>(
+                    8, std::min<int64_t>((A.m + 255) / 256, (int64_t)sms * 8));
+                hist_logprod_init_kernel<<<gi, 256, 0, s>>>(A.hdr, G, A.tab);
+                const int hot = (int)std::min<int64_t>(A.m, kLogHot);
+                const int H = (int)std::min<int64_t>(A.m, kLogHot + kLogSlots);
+                const size_t sh = kLogTab * 16 + (size_t)(31 * hot + H) * 16;
+                const int gp = (int)std::max<int64_t>(
+                    1, std::min<int64_t>((A.n + 4 * kLogThreads - 1) / (4 * kLogThreads), sms));
+                hist_logprod_kernel<I><<<gp, kLogThreads, sh, s>>>(G);
+                const bool map = !A.primal_only && !A.logdomain && A.n > 0;
+                hist_logprod_bins_kernel<<<gridM, 256, 0, s>>>(G, static_cast<const float*>(A.hsbar),
+                                                               map ? A.binq : nullptr,
+                                                               static_cast<float*>(A.hs_out), A.bin_aux,
+                                                               A.logdomain);
+                if (map) {
+                    const int g = (int)std::max<int64_t>(
+                        1, std::min<int64_t>((A.n / 4 + 255) / 256, (int64_t)sms * 8));
+                    hist_logprod_vjp_kernel<I><<<g, 256, 0, s>>>(G, A.binq, static_cast<float*>(A.valsbar),
+                                                                 A.accumulate);
+                } else if (!A.primal_only) {
+                    hist_prod_vjp_kernel<T, I><<<gridN, kHistBlock, 0, s>>>(A);
+                }
+                break;
+            }
+        }
         const int64_t h1 = std::min<int64_t>(A.m, kProdWarpBins);
         const int64_t h2 = std::max<int64_t>(0, std::min<int64_t>(A.m - h1, kProdBlockBins));
         const size_t sh = (size_t)h1 * 24 * (kProdBlock / 32) + (size_t)h2 * 28;
@@ -838,15 +679,10 @@ int run_hist(HistArgs A, cudaStream_t s) {
             1, std::min<int64_t>((A.n + kProdBlock - 1) / kProdBlock, std::min<int64_t>(sms * 4, kProdMaxGrid)));
         A.hw = h1 + h2;
         hist_prod_kernel<T, I><<<gridP, kProdBlock, sh, s>>>(A);
-        if (A.hw > 0) hist_prod_merge_kernel<T><<<(unsigned)((A.hw * 32 + 255) / 256), 256, 0, s>>>(A, gridP);
+        if (A.hw > 0) hist_prod_merge_kernel<<<(unsigned)((A.hw * 32 + 255) / 256), 256, 0, s>>>(A, gridP);
         if (A.hs_out || A.bin_aux) hist_prod_bins_kernel<T><<<gridM, 256, 0, s>>>(A);
         if (A.primal_only) break;
-        if (sizeof(T) == 4 && !A.logdomain) {
-            hist_prod_binq_kernel<T><<<gridM, 256, 0, s>>>(A);
-            hist_prod_vjp_f32_kernel<I><<<gridN, kHistBlock, 0, s>>>(A);
-        } else {
-            hist_prod_vjp_kernel<T, I><<<gridN, kHistBlock, 0, s>>>(A);
-        }
+        hist_prod_vjp_kernel<T, I><<<gridN, kHistBlock, 0, s>>>(A);
         break;
     }
     default:
@@ -864,6 +700,7 @@ void configure_smem() {
     cudaFuncSetAttribute(hist_add_primal_kernel<T, I>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024);
     cudaFuncSetAttribute(hist_prod_kernel<T, I>, cudaFuncAttributeMaxDynamicSharedMemorySize, 112 * 1024);
     if constexpr (sizeof(T) == 4) {
+        cudaFuncSetAttribute(hist_logprod_kernel<I>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLogSmem);
         cudaFuncSetAttribute(hist_arg_f32_kernel<I, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024);
         cudaFuncSetAttribute(hist_arg_f32_kernel<I, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024);
     }
@@ -871,11 +708,11 @@ void configure_smem() {
 
 }  // namespace
 
-size_t hist_workspace_size(adpar_opdesc d, int64_t m) {
+size_t hist_workspace_size(adpar_opdesc d, int64_t n, int64_t m) {
     if (m < 0 || (d.dtype != ADPAR_F32 && d.dtype != ADPAR_F64)) return (size_t)-1;
     if (d.op != ADPAR_OP_ADD && d.op != ADPAR_OP_MUL && d.op != ADPAR_OP_MIN && d.op != ADPAR_OP_MAX)
         return (size_t)-1;
-    return hist_layout(d.op, d.dtype, m).total;
+    return hist_layout(d.op, d.dtype, n, m).total;
 }
 
 }  // namespace adpar
@@ -904,7 +741,7 @@ int hist_impl(adpar_opdesc d, int64_t n, int64_t m, const void* vals, const void
     const void* ptrs[] = {vals, inds, hsbar, valsbar, hs_out};
     for (const void* p : ptrs)
         if (p && !aligned16(p)) return ADPAR_ERR_ALIGN;
-    const HistLayout L = hist_layout(d.op, d.dtype, m);
+    const HistLayout L = hist_layout(d.op, d.dtype, n, m);
     if (!work || work_bytes < L.total || (reinterpret_cast<uintptr_t>(work) & 255u)) return ADPAR_ERR_WORKSPACE;
     if (n == 0 && m == 0) return ADPAR_OK;
     HistArgs A{};
@@ -928,15 +765,20 @@ int hist_impl(adpar_opdesc d, int64_t n, int64_t m, const void* vals, const void
     if (L.off_idx) A.idx = reinterpret_cast<unsigned long long*>(w + L.off_idx);
     if (L.off_binq) A.binq = reinterpret_cast<BinQ*>(w + L.off_binq);
     if (L.off_part_m) {
-        A.part_m = reinterpret_cast<unsigned long long*>(w + L.off_part_m);
+        A.part_m = reinterpret_cast<double*>(w + L.off_part_m);
         A.part_e = reinterpret_cast<long long*>(w + L.off_part_e);
         A.part_f = reinterpret_cast<long long*>(w + L.off_part_f);
         A.part_z = reinterpret_cast<unsigned*>(w + L.off_part_z);
     }
-    A.q62 = (d.op == ADPAR_OP_MUL && d.dtype == ADPAR_F32) ? 1 : 0;
+    if (L.off_acc) {
+        A.acc = reinterpret_cast<ulonglong2*>(w + L.off_acc);
+        A.tab = reinterpret_cast<ulonglong2*>(w + L.off_tab);
+    }
     if (L.off_pm) {
         A.pm = reinterpret_cast<double*>(w + L.off_pm);
         A.pe = reinterpret_cast<long long*>(w + L.off_pe);
+    }
+    if (L.off_pz) {
         A.pz = reinterpret_cast<unsigned int*>(w + L.off_pz);
         A.pf = reinterpret_cast<long long*>(w + L.off_pf);
     }
