@@ -26,41 +26,134 @@ __device__ __forceinline__ int64_t ldi(const I* p, int64_t j) {
     return (int64_t)__ldcs(p + j);
 }
 
-// Four indices per thread per step: the four random reads (and then the
-// four random zeroing writes) are independent, so each thread keeps four
-// scattered accesses in flight instead of one dependent chain.
-template <class T, class I>
-__global__ void __launch_bounds__(kBlk) scatter_vjp_kernel(int64_t n, int64_t m, const I* is, T* ysbar,
-                                                          T* vsbar, T* ys, const T* xs_saved, int accumulate) {
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x * 4;
-    for (int64_t j0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) * 4; j0 < m; j0 += stride) {
-        const int cnt = (int)(m - j0 < 4 ? m - j0 : 4);
-        int64_t k[4];
-        bool in[4];
-        T g[4];
+// Random accesses to an array larger than L2 cost a DRAM fetch and a write-back
+// per index (32 bytes and more of each for 4 useful ones).  So a large target is
+// taken in regions that L2 holds, last region first (what a preceding copy wrote
+// last): every thread goes through its indices once per region and touches only
+// those in it, so a line is fetched and written back once for all of its
+// indices, at the price of reading the indices once per region.
+// Worth it when a 64-byte line holds an index or more on average (below, nothing
+// is shared) and for 8 regions at most (16: 6.7 ms against 5.2 ms in one, 2^26
+// indices into 1 GB); not when the indices are local already (sorted, say):
+// each block looks at 256 pairs 64 apart, the same pairs in all blocks, and
+// takes one region when most lie close.
+// Random accesses of 4 bytes on a GB300, in G/s, within 64 MB / over 256 MB:
+// loads 286 / 77, stores 209 / 33, exchanges 134 / 36.  Forward and VJP through
+// autograd, 2^24 indices into 2^26 FP32 (of it 170 us for the two copies of the
+// target): 1557 us with a load and a store per index in one region, 741 us so;
+// regions of 32 and 90 MB 1190 and 865 us.
+constexpr int64_t kRegionBytes = int64_t(64) << 20;
+constexpr int64_t kMaxRegions = 8;
+constexpr int64_t kLocalBytes = int64_t(1) << 20;
+// blocks per SM, all resident: the grid goes through the regions together
+constexpr int kScatBlocks = 6;
+
+// elements per region (below 2^32): all of n where one region will do
+inline int64_t region_elems(int64_t n, int64_t m, size_t esz) {
+    const int64_t bytes = n * (int64_t)esz;
+    const int64_t regions = (bytes + kRegionBytes - 1) / kRegionBytes;
+    if (bytes < 2 * kRegionBytes || regions > kMaxRegions || m < 4096 || m * 64 < bytes)
+        return std::min<int64_t>(std::max<int64_t>(n, 1), int64_t(1) << 31);
+    return ((n + regions - 1) / regions + 31) / 32 * 32;
+}
+
+// the region size this launch uses (the same in every block); all threads call it
+template <class I>
+__device__ __forceinline__ int64_t pick_region(const I* is, int64_t n, int64_t m, int64_t region, int esz) {
+    if (region >= n || region == int64_t(1) << 31) return region;
+    const int64_t p = (int64_t)threadIdx.x * ((m - 64) / blockDim.x);
+    const int64_t d = (int64_t)is[p + 64] - (int64_t)is[p];
+    const int near = __syncthreads_count((d < 0 ? -d : d) <= kLocalBytes / esz);
+    return 2 * near >= (int)blockDim.x ? (n < (int64_t(1) << 31) ? n : int64_t(1) << 31) : region;
+}
+
+// Asks L2 for a region's lines in order, each block for its share, ahead of the
+// random accesses (which would fetch them one 32-byte sector at a time).
+template <class T>
+__device__ __forceinline__ void prefetch_region(const T* p, unsigned size) {
+    const char* lo = reinterpret_cast<const char*>(p);
+    const int64_t bytes = (int64_t)size * (int64_t)sizeof(T) / 16 * 16;
+    const int64_t share = (bytes / gridDim.x / 512 + 1) * 512, first = share * blockIdx.x;
+    const int64_t stop = first + share < bytes ? first + share : bytes;
+    for (int64_t o = first + threadIdx.x * 512; o < stop; o += kBlk * 512) {
+        const unsigned sz = (unsigned)(stop - o < 512 ? stop - o : 512);
+        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(lo + o), "r"(sz) : "memory");
+    }
+}
+
+// Puts v at p and returns what was there, in one trip to L2.  A load and then a
+// store to a random line is far slower (26 against 36 G/s beyond L2, 62 against
+// 134 within): the line's copy on the reading die's side of L2 is made and
+// thrown away again.
+__device__ __forceinline__ float exchange(float* p, float v) { return atomicExch(p, v); }
+__device__ __forceinline__ double exchange(double* p, double v) {
+    return __longlong_as_double((long long)atomicExch(reinterpret_cast<unsigned long long*>(p),
+                                                      (unsigned long long)__double_as_longlong(v)));
+}
+template <class T>
+__device__ __forceinline__ T take_zero(T* p) {
+    return exchange(p, T(0));
+}
+
+// Four indices per thread and step, a block apart (neighbouring lanes hold
+// neighbouring indices).  Loading the next step's ahead loses (800 against 741 us
+// below): the more index lines in flight, the fewer of the region's stay in L2.
+constexpr int kScatU = 4;
+
+// fn(r, j) for every index j of this thread whose target lies in [base, base + size),
+// r its offset there; out(j) for those outside [0, n).  OUT: call out().
+template <bool OUT, class I, class Fn, class Out>
+__device__ __forceinline__ void for_region(const I* is, int64_t m, int64_t n, int64_t base, unsigned size, Fn fn,
+                                           Out out) {
+    constexpr int U = kScatU;
+    const int64_t stride = (int64_t)gridDim.x * (kBlk * U);
+    for (int64_t j = blockIdx.x * (int64_t)(kBlk * U) + threadIdx.x; j < m; j += stride) {
+        I q[U];
+        unsigned r[U];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            k[u] = u < cnt ? ldi(is, j0 + u) : -1;
-            in[u] = k[u] >= 0 && k[u] < n;
+        for (int u = 0; u < U; ++u) q[u] = j + u * kBlk < m ? __ldcs(is + j + u * kBlk) : I(-1);
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int64_t k = (int64_t)q[u], d = k - base;
+            r[u] = (unsigned long long)d < size ? (unsigned)d : 0xffffffffu;
+            if (OUT && (k < 0 || k >= n) && j + u * kBlk < m) out(j + u * kBlk);
         }
+        fn(r, j);
+    }
+}
+
+template <class T, class I, bool RESTORE, bool ACC>
+__global__ void __launch_bounds__(kBlk, kScatBlocks) scatter_vjp_kernel(int64_t n, int64_t m, const I* is, T* ysbar,
+                                                                       T* vsbar, T* ys, const T* xs_saved,
+                                                                       int64_t region_arg) {
+    constexpr int U = kScatU;
+    const int64_t region = pick_region(is, n, m, region_arg, (int)sizeof(T));
+    const int64_t last = n > 0 ? (n - 1) / region * region : 0;
+    for (int64_t base = last; base >= 0; base -= region) {
+        const int64_t left = n - base;
+        const unsigned size = (unsigned)(left < region ? left : region);
+        if (region < n && region <= kRegionBytes) prefetch_region(ysbar + base, size);
+        T* yb = ysbar + base;
+        auto fn = [&](const unsigned (&r)[U], int64_t j) {
+            T g[U];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) g[u] = in[u] ? ysbar[k[u]] : T(0);
+            for (int u = 0; u < U; ++u) g[u] = r[u] != 0xffffffffu ? take_zero(yb + r[u]) : T(0);
+            if (RESTORE) {
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            if (in[u]) {
-                ysbar[k[u]] = T(0);
-                if (ys) ys[k[u]] = __ldcs(xs_saved + j0 + u);
+                for (int u = 0; u < U; ++u)
+                    if (r[u] != 0xffffffffu) ys[base + r[u]] = __ldcs(xs_saved + j + u * kBlk);
             }
-        }
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            if (u >= cnt) break;
-            if (accumulate) {
-                if (in[u]) vsbar[j0 + u] += g[u];
-            } else {
-                __stcs(vsbar + j0 + u, g[u]);
+            for (int u = 0; u < U; ++u) {
+                T* o = vsbar + j + u * kBlk;
+                if (r[u] != 0xffffffffu) __stcs(o, ACC ? __ldcs(o) + g[u] : g[u]);
             }
-        }
+        };
+        // an index out of range: vsbar 0 (overwrite), in the first region's pass
+        if (!ACC && base == last)
+            for_region<true>(is, m, n, base, size, fn, [&](int64_t j) { vsbar[j] = T(0); });
+        else
+            for_region<false>(is, m, n, base, size, fn, [](int64_t) {});
     }
 }
 
@@ -138,19 +231,33 @@ __global__ void __launch_bounds__(kBlk) map_acc_kernel(MapAccArgs<T> A) {
 }
 
 // primal of scatter (Sec. 5.3's forward sweep): xs_saved[j] = ys[is_j]
-// (optional), then ys[is_j] = vs[j], in place
-template <class T, class I>
-__global__ void __launch_bounds__(kBlk) scatter_fwd_kernel(int64_t n, int64_t m, const I* is, const T* vs, T* ys,
-                                                          T* xs_saved) {
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < m; j += stride) {
-        const int64_t k = ldi(is, j);
-        if (k < 0 || k >= n) {
-            if (xs_saved) xs_saved[j] = T(0);
-            continue;
-        }
-        if (xs_saved) xs_saved[j] = ys[k];
-        ys[k] = __ldcs(vs + j);
+// (optional), then ys[is_j] = vs[j], in place; by regions as above
+template <class T, class I, bool SAVE>
+__global__ void __launch_bounds__(kBlk, kScatBlocks) scatter_fwd_kernel(int64_t n, int64_t m, const I* is, const T* vs,
+                                                                       T* ys, T* xs_saved, int64_t region_arg) {
+    constexpr int U = kScatU;
+    const int64_t region = pick_region(is, n, m, region_arg, (int)sizeof(T));
+    const int64_t last = n > 0 ? (n - 1) / region * region : 0;
+    for (int64_t base = last; base >= 0; base -= region) {
+        const int64_t left = n - base;
+        const unsigned size = (unsigned)(left < region ? left : region);
+        if (region < n && region <= kRegionBytes) prefetch_region(ys + base, size);
+        T* y = ys + base;
+        auto fn = [&](const unsigned (&r)[U], int64_t j) {
+            T g[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) g[u] = r[u] != 0xffffffffu ? __ldcs(vs + j + u * kBlk) : T(0);
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                if (r[u] == 0xffffffffu) continue;
+                if (SAVE) xs_saved[j + u * kBlk] = exchange(y + r[u], g[u]);
+                else y[r[u]] = g[u];
+            }
+        };
+        if (SAVE && base == last)
+            for_region<true>(is, m, n, base, size, fn, [&](int64_t j) { xs_saved[j] = T(0); });
+        else
+            for_region<false>(is, m, n, base, size, fn, [](int64_t) {});
     }
 }
 
@@ -212,19 +319,24 @@ extern "C" int adpar_vjp_scatter(int dtype, int64_t n, int64_t m, const void* is
         if (p && !aligned16(p)) return ADPAR_ERR_ALIGN;
     if (m == 0) return ADPAR_OK;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((m / 4 + kBlk) / kBlk, (int64_t)sm_count() * 8));
+    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((m / kScatU + kBlk) / kBlk, (int64_t)sm_count() * kScatBlocks));
+    const int64_t region = region_elems(n, m, dtype == ADPAR_F64 ? 8 : 4);
     const int acc = (flags & ADPAR_ACCUMULATE) ? 1 : 0;
     void* ys = restore ? ys_restore : nullptr;
-#define ADPAR_SCATTER(T, I)                                                                               \
-    scatter_vjp_kernel<T, I><<<grid, kBlk, 0, s>>>(n, m, static_cast<const I*>(is), static_cast<T*>(ysbar_inout), \
-                                                   static_cast<T*>(vsbar), static_cast<T*>(ys),              \
-                                                   static_cast<const T*>(xs_saved), acc)
+#define ADPAR_SCATTER_RA(T, I, R, A)                                                                             \
+    scatter_vjp_kernel<T, I, R, A><<<grid, kBlk, 0, s>>>(n, m, static_cast<const I*>(is), static_cast<T*>(ysbar_inout), \
+                                                         static_cast<T*>(vsbar), static_cast<T*>(ys),            \
+                                                         static_cast<const T*>(xs_saved), region)
+#define ADPAR_SCATTER(T, I)                                                                                 \
+    (ys ? (acc ? ADPAR_SCATTER_RA(T, I, true, true) : ADPAR_SCATTER_RA(T, I, true, false))                  \
+        : (acc ? ADPAR_SCATTER_RA(T, I, false, true) : ADPAR_SCATTER_RA(T, I, false, false)))
     if (dtype == ADPAR_F32) {
         if (itype == ADPAR_I32) ADPAR_SCATTER(float, int32_t); else ADPAR_SCATTER(float, int64_t);
     } else {
         if (itype == ADPAR_I32) ADPAR_SCATTER(double, int32_t); else ADPAR_SCATTER(double, int64_t);
     }
 #undef ADPAR_SCATTER
+#undef ADPAR_SCATTER_RA
     return cudaGetLastError() == cudaSuccess ? ADPAR_OK : ADPAR_ERR_CUDA;
 }
 
@@ -290,16 +402,19 @@ extern "C" int adpar_scatter(int dtype, int64_t n, int64_t m, const void* is, in
         if (p && !aligned16(p)) return ADPAR_ERR_ALIGN;
     if (m == 0) return ADPAR_OK;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((m + kBlk - 1) / kBlk, (int64_t)sm_count() * 8));
-#define ADPAR_SCAT_FWD(T, I)                                                                                   \
-    scatter_fwd_kernel<T, I><<<grid, kBlk, 0, s>>>(n, m, static_cast<const I*>(is), static_cast<const T*>(vs), \
-                                                   static_cast<T*>(ys_inout), static_cast<T*>(xs_saved_out))
+    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((m / kScatU + kBlk) / kBlk, (int64_t)sm_count() * kScatBlocks));
+    const int64_t region = region_elems(n, m, dtype == ADPAR_F64 ? 8 : 4);
+#define ADPAR_SCAT_FWD_S(T, I, S)                                                                                 \
+    scatter_fwd_kernel<T, I, S><<<grid, kBlk, 0, s>>>(n, m, static_cast<const I*>(is), static_cast<const T*>(vs), \
+                                                      static_cast<T*>(ys_inout), static_cast<T*>(xs_saved_out), region)
+#define ADPAR_SCAT_FWD(T, I) (xs_saved_out ? ADPAR_SCAT_FWD_S(T, I, true) : ADPAR_SCAT_FWD_S(T, I, false))
     if (dtype == ADPAR_F32) {
         if (itype == ADPAR_I32) ADPAR_SCAT_FWD(float, int32_t); else ADPAR_SCAT_FWD(float, int64_t);
     } else {
         if (itype == ADPAR_I32) ADPAR_SCAT_FWD(double, int32_t); else ADPAR_SCAT_FWD(double, int64_t);
     }
 #undef ADPAR_SCAT_FWD
+#undef ADPAR_SCAT_FWD_S
     return cudaGetLastError() == cudaSuccess ? ADPAR_OK : ADPAR_ERR_CUDA;
 }
 
