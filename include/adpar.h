@@ -634,6 +634,13 @@ int adpar_hist(adpar_opdesc desc, int64_t n, int64_t m, const void *vals, const 
                void *hs_out, int64_t *argidx_out, adpar_prod_aux *bin_aux_out, void *work,
                size_t work_bytes, void *stream);
 
+/* hs = reduce_by_index (.) inds (a, b) for any operator of
+ * adpar_vjp_hist_general (LINREC among them: the recurrence over a bin's
+ * elements in index order), into hs_a [m] (and hs_b [m] for LINREC), required.
+ * Arguments, limits and workspace as for adpar_vjp_hist_general. */
+int adpar_hist_general(adpar_opdesc desc, int64_t n, int64_t m, const void *a, const void *b, const void *inds,
+                       int itype, void *hs_a, void *hs_b, void *work, size_t work_bytes, void *stream);
+
 /* ys = scatter ys is vs in place (ys_inout [n] holds xs on entry), saving
  * the overwritten values xs_saved_out[j] = xs[is_j] first (nullable), the
  * forward sweep of Sec. 5.3.  Out-of-range indices are skipped. */

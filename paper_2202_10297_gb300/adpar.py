@@ -129,6 +129,7 @@ def _bind_optional(L):
         "adpar_kmeans_fwd_rev": [C.c_int64, C.c_int, C.c_int, _VP, _VP, _VP, _VP, _VP, _VP, C.c_uint32, _VP,
                                  C.c_size_t, _VP],
         "adpar_hist": [OpDesc, C.c_int64, C.c_int64, _VP, _VP, C.c_int, _VP, _VP, _VP, _VP, C.c_size_t, _VP],
+        "adpar_hist_general": [OpDesc, C.c_int64, C.c_int64, _VP, _VP, _VP, C.c_int, _VP, _VP, _VP, C.c_size_t, _VP],
         "adpar_scatter": [C.c_int, C.c_int64, C.c_int64, _VP, C.c_int, _VP, _VP, _VP, _VP],
         "adpar_map_acc": [C.c_int, C.c_int, C.c_int64, C.c_int64, C.c_int, _VP, _VP, C.c_int, _VP, _VP, _VP],
     }
@@ -661,6 +662,28 @@ def adpar_hist(op, vals, inds, m, want_argidx=False, work=None, stream=None):
     _check("adpar_hist", lib().adpar_hist(OpDesc(opc, dt, 1), n, m, _ptr(vals), _ptr(inds), _itype_code(inds),
                                           _ptr(hs), _ptr(arg), None, _ptr(work), work.numel(), _stream(stream)))
     return hs, arg
+
+
+def adpar_hist_general(op, a, inds, m, b=None, work=None, stream=None):
+    """Primal reduce_by_index of any operator, LINREC included (C: adpar_hist_general).
+    Returns (hs_a [m], hs_b [m] or None)."""
+    opc = OPS[op] if isinstance(op, str) else int(op)
+    n = a.numel()
+    dt = _dtype_code(a)
+    w = 2 if opc == OP_LINREC else 1
+    if b is not None and (b.dtype != a.dtype or b.numel() != n):
+        raise ValueError("all element arrays must share dtype and length")
+    if inds.numel() != n:
+        raise ValueError("inds must have one index per element")
+    hs_a = torch.empty(m, dtype=a.dtype, device=a.device)
+    hs_b = torch.empty(m, dtype=a.dtype, device=a.device) if w == 2 else None
+    need = adpar_workspace_size(RULE_HIST_GENERAL, opc, dt, n, m)
+    if work is None or work.numel() < need:
+        work = workspace(need, a.device)
+    _check("adpar_hist_general", lib().adpar_hist_general(OpDesc(opc, dt, w), n, m, _ptr(a), _ptr(b), _ptr(inds),
+                                                          _itype_code(inds), _ptr(hs_a), _ptr(hs_b), _ptr(work),
+                                                          work.numel(), _stream(stream)))
+    return hs_a, hs_b
 
 
 def adpar_scatter(is_, vs, ys_inout, xs_saved=None, stream=None):

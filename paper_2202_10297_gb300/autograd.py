@@ -116,14 +116,11 @@ class _Hist(torch.autograd.Function):
 
 
 class _HistGeneral(torch.autograd.Function):
-    """reduce_by_index by the general rule (radix sort by bin, segmented
-    scans); its forward is the same call with a zero cotangent, which
-    recomputes the bins."""
+    """reduce_by_index by the general rule (radix sort by bin, segmented scans)."""
 
     @staticmethod
     def forward(ctx, op, a, b, inds, m):
-        z = torch.zeros(m, dtype=a.dtype, device=a.device)
-        _, _, hs_a, hs_b = A.adpar_vjp_hist_general(op, a, inds, m, z, b=b, hsbar_b=z, want_hs=True)
+        hs_a, hs_b = A.adpar_hist_general(op, a, inds, m, b=b)
         ctx.op, ctx.m = op, m
         ctx.save_for_backward(a, b, inds)
         return hs_a, hs_b

@@ -35,15 +35,21 @@
 namespace adpar {
 namespace {
 
-constexpr int kSortBlock = 256;
+constexpr int kSortBlock = 512;
 constexpr int kSortNW = kSortBlock / 32;
-// elements per thread and tile of the scatter (a tile is staged in static
-// shared memory: fewer for FP64 pairs)
+// Elements per thread and tile of the scatter, staged in shared memory.  A tile's
+// run of one digit is about TILE / 256 elements; a run that ends inside a 32-byte
+// sector costs a partial-sector write, so long arrays take large tiles, short
+// ones small tiles on more blocks.  10 per thread (5120 elements) is what 64
+// registers hold, with two blocks an SM: forward and backward of 2^24 LINREC
+// elements in 2^16 Zipf bins 1152 us; 12: 1204, 16: 1325 (spills), 8 with three
+// blocks: 1460.
+constexpr int kBigItems = 10, kSmallItems = 4;
 template <class T, int W>
-constexpr int sort_items() {
-    return sizeof(T) == 8 && W == 2 ? 6 : 8;
+constexpr int big_items() {
+    return sizeof(T) == 8 && W == 2 ? 6 : kBigItems;
 }
-constexpr int kChunkAlign = kSortBlock * 24;  // a multiple of every tile
+constexpr int64_t kBigSort = int64_t(1) << 21;  // elements from which tiles are large
 constexpr int kRadixBits = 8;
 constexpr int kRadix = 1 << kRadixBits;
 constexpr int kSortMaxGrid = 2048;
@@ -53,18 +59,40 @@ constexpr int kSegK = 2;  // chunks per tile
 constexpr int kSegTile = kSegK * kSegBlock * kSegV;
 constexpr uint32_t kNoKey = 0xffffffffu;  // above every bin number (m < 2^31)
 
-// ------------------------------------------------------------ radix sort
+// One element's values: the pair (a, b) of LINREC side by side, so that a
+// scattered element is one store and a gathered one one load.
+template <class T, int W>
+struct alignas(W * sizeof(T)) Elem {
+    T a, b;
+};
 template <class T>
+struct Elem<T, 1> {
+    T a;
+};
+template <class T, int W>
+__device__ __forceinline__ Elem<T, W> make_elem(T a, T b) {
+    if constexpr (W == 2) return Elem<T, W>{a, b};
+    else return Elem<T, W>{a};
+}
+template <class T, int W>
+__device__ __forceinline__ T elem_b(const Elem<T, W>& e) {
+    if constexpr (W == 2) return e.b;
+    else return T(0);
+}
+
+// ------------------------------------------------------------ radix sort
+template <class T, int W>
 struct SortPass {
     int64_t n, m;          // all elements; bins
-    const void* inds;      // first pass: the caller's indices
+    const void* inds;      // first pass: the caller's indices and values
+    const T* a;
+    const T* b;
     const uint32_t* kin;   // later passes: keys and values
-    const T* ain;
-    const T* bin;
+    const Elem<T, W>* ein;
     uint32_t* kout;
-    T* aout;
-    T* bout;
-    uint32_t* dest;        // [input length] where each input element went (kNoKey: left the sort)
+    Elem<T, W>* eout;
+    uint32_t* dest;        // [input length] where each input element went (kNoKey: left the
+                           // sort); NULL when nothing is returned to the input order
     uint32_t* cnt;         // [2^bits][G] digit counts per block, then their exclusive scan
     uint32_t* rowtot;      // [2^bits] elements per digit
     const uint32_t* nsorted;  // in-range elements (set by the first pass)
@@ -73,9 +101,9 @@ struct SortPass {
 
 // Block c of a pass covers [c * len_c, (c + 1) * len_c) of its input, a
 // whole number of tiles.
-__device__ __forceinline__ int64_t block_chunk(int64_t len, int G) {
+__host__ __device__ __forceinline__ int64_t block_chunk(int64_t len, int G, int tile) {
     const int64_t c = (len + G - 1) / G;
-    return (c + kChunkAlign - 1) / kChunkAlign * kChunkAlign;
+    return (c + tile - 1) / tile * tile;
 }
 
 // Exclusive scan of one value per thread over a block of kSortBlock.
@@ -105,8 +133,8 @@ __device__ __forceinline__ uint32_t block_excl_u32(uint32_t x, uint32_t* s_w, ui
     return r;
 }
 
-template <class I, class T, bool FIRST>
-__device__ __forceinline__ bool sort_key(const SortPass<T>& P, int64_t i, uint32_t& key) {
+template <class I, class T, int W, bool FIRST>
+__device__ __forceinline__ bool sort_key(const SortPass<T, W>& P, int64_t i, uint32_t& key) {
     if constexpr (FIRST) {
         const int64_t ix = (int64_t)static_cast<const I*>(P.inds)[i];
         key = (uint32_t)ix;
@@ -117,20 +145,30 @@ __device__ __forceinline__ bool sort_key(const SortPass<T>& P, int64_t i, uint32
     }
 }
 
-template <class I, class T, bool FIRST>
-__global__ void __launch_bounds__(kSortBlock) hg_count_kernel(SortPass<T> P) {
+template <class I, class T, int W, bool FIRST>
+__global__ void __launch_bounds__(kSortBlock) hg_count_kernel(SortPass<T, W> P, int tile) {
     __shared__ uint32_t h[kSortNW][kRadix];
     const int warp = threadIdx.x >> 5;
     for (int q = threadIdx.x; q < kSortNW * kRadix; q += kSortBlock) (&h[0][0])[q] = 0u;
     __syncthreads();
     const int64_t len = FIRST ? P.n : (int64_t)*P.nsorted;
-    const int64_t bc = block_chunk(len, P.G);
+    const int64_t bc = block_chunk(len, P.G, tile);
     const int64_t lo = (int64_t)blockIdx.x * bc;
     const int64_t hi = lo + bc < len ? lo + bc : len;
     const uint32_t dmask = (1u << P.bits) - 1u;
-    for (int64_t i = lo + threadIdx.x; i < hi; i += kSortBlock) {
+    int64_t i = lo + threadIdx.x;
+    for (; i + 3 * kSortBlock < hi; i += 4 * kSortBlock) {
+        uint32_t key[4];
+        bool ok[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) ok[u] = sort_key<I, T, W, FIRST>(P, i + u * kSortBlock, key[u]);
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (ok[u]) atomicAdd(&h[warp][(key[u] >> P.shift) & dmask], 1u);
+    }
+    for (; i < hi; i += kSortBlock) {
         uint32_t key;
-        if (sort_key<I, T, FIRST>(P, i, key)) atomicAdd(&h[warp][(key >> P.shift) & dmask], 1u);
+        if (sort_key<I, T, W, FIRST>(P, i, key)) atomicAdd(&h[warp][(key >> P.shift) & dmask], 1u);
     }
     __syncthreads();
     for (int d = threadIdx.x; d < (1 << P.bits); d += kSortBlock) {
@@ -175,73 +213,95 @@ __global__ void __launch_bounds__(kSortBlock) hg_scan_counts_kernel(uint32_t* cn
     }
 }
 
-// Stable scatter of one pass.  A block takes its chunk tile by tile (warp
-// w holds the tile's elements [w*256, (w+1)*256), 32 consecutive ones per
-// item).  Every element gets its rank among the equal digits before it in
-// the tile (the lanes of equal digit from one ballot per digit bit, per-warp
-// digit counts, their scan over the warps
-// and the digits), which is its place in the tile sorted by digit; the tile
-// is staged in that order in shared memory and written out so that each
-// digit's run lands contiguously after the block's previous run of that
-// digit.  Blocks and tiles are in input order and the counts were scanned
-// over the blocks digit by digit, so equal digits keep their input order.
-template <class I, class T, int W, bool FIRST>
-__global__ void __launch_bounds__(kSortBlock) hg_scatter_kernel(SortPass<T> P) {
-    constexpr int kSortItems = sort_items<T, W>();
-    constexpr int kSortTile = kSortBlock * kSortItems;
-    __shared__ uint32_t s_cnt[kSortNW][kRadix];
-    __shared__ uint32_t s_off[kRadix];    // the block's next global position per digit
-    __shared__ uint32_t s_start[kRadix];  // the digit's first place in the sorted tile
-    __shared__ uint32_t s_w[kSortNW + 1];
-    __shared__ uint32_t s_key[kSortTile];
-    __shared__ T s_a[kSortTile];
-    __shared__ T s_b[W == 2 ? kSortTile : 1];
+__device__ __forceinline__ void prefetch_l2(const void* p) {
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
+}
+
+template <class T, int W, int ITEMS>
+constexpr size_t sort_smem() {
+    return (size_t)kSortBlock * ITEMS * (sizeof(Elem<T, W>) + 4) + kSortNW * kRadix * 2 + 2 * kRadix * 4 +
+           (kSortNW + 1) * 4;
+}
+
+// Stable scatter of one pass.  A block takes its chunk tile by tile (warp w
+// holds the tile's elements [w * 32 ITEMS, (w + 1) * 32 ITEMS), 32 consecutive
+// ones per item).  Every element gets its rank among the equal digits before
+// it in the tile (the lanes of equal digit from one ballot per digit bit,
+// per-warp digit counts, their scan over the warps and the digits), which is
+// its place in the tile sorted by digit; the tile is staged in that order in
+// shared memory and written out so that each digit's run lands contiguously
+// after the block's previous run of that digit.  Blocks and tiles are in input
+// order and the counts were scanned over the blocks digit by digit, so equal
+// digits keep their input order.
+template <class I, class T, int W, bool FIRST, int ITEMS>
+__global__ void __launch_bounds__(kSortBlock, 2) hg_scatter_kernel(SortPass<T, W> P) {
+    constexpr int kTile = kSortBlock * ITEMS;
+    using E = Elem<T, W>;
+    extern __shared__ __align__(16) unsigned char s_dyn[];
+    E* s_e = reinterpret_cast<E*>(s_dyn);
+    uint32_t* s_key = reinterpret_cast<uint32_t*>(s_e + kTile);
+    uint32_t* s_off = s_key + kTile;     // [kRadix] the block's next global position per digit
+    uint32_t* s_start = s_off + kRadix;  // [kRadix] the digit's first place in the sorted tile
+    uint32_t* s_w = s_start + kRadix;    // [kSortNW + 1]
+    uint16_t* s_cnt = reinterpret_cast<uint16_t*>(s_w + kSortNW + 1);  // [kSortNW][kRadix]
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int R = 1 << P.bits;
     const uint32_t dmask = (uint32_t)R - 1u;
+    uint16_t* my_cnt = s_cnt + warp * kRadix;
     {
         const uint32_t rt = threadIdx.x < R ? P.rowtot[threadIdx.x] : 0u;
         const uint32_t ex = block_excl_u32(rt, s_w);
         if (threadIdx.x < R) s_off[threadIdx.x] = ex + P.cnt[(int64_t)threadIdx.x * P.G + blockIdx.x];
     }
     const int64_t len = FIRST ? P.n : (int64_t)*P.nsorted;
-    const int64_t bc = block_chunk(len, P.G);
+    const int64_t bc = block_chunk(len, P.G, kTile);
     const int64_t lo = (int64_t)blockIdx.x * bc;
     const int64_t hi = lo + bc < len ? lo + bc : len;
     const uint32_t lt = (1u << lane) - 1u;
-    for (int64_t t0 = lo; t0 < hi; t0 += kSortTile) {
-        for (int q = threadIdx.x; q < kSortNW * kRadix; q += kSortBlock) (&s_cnt[0][0])[q] = 0u;
-        __syncthreads();
-        uint32_t key[kSortItems], rk[kSortItems];
-        T va[kSortItems], vb[kSortItems];
-        bool ok[kSortItems];
-#pragma unroll
-        for (int u = 0; u < kSortItems; ++u) {
-            const int64_t i = t0 + warp * (32 * kSortItems) + u * 32 + lane;
-            ok[u] = false;
-            key[u] = 0u;
-            va[u] = T(0);
-            vb[u] = T(0);
-            if (i < hi) {  // values loaded beside the key, not after its range test
-                ok[u] = sort_key<I, T, FIRST>(P, i, key[u]);
-                va[u] = __ldcs(P.ain + i);
-                if constexpr (W == 2) vb[u] = __ldcs(P.bin + i);
-            }
+    // the values of the tile at t into L2, while its keys are ranked (asking for
+    // the next tile, or for the keys too, measured no better)
+    auto prefetch_tile = [&](int64_t t) {
+        const int64_t cnt = hi - t < kTile ? hi - t : kTile;
+        auto lines = [&](const void* p, int64_t bytes) {
+            for (int64_t o = threadIdx.x * 128; o < bytes; o += kSortBlock * 128)
+                prefetch_l2(static_cast<const char*>(p) + o);
+        };
+        if constexpr (FIRST) {
+            lines(P.a + t, cnt * (int64_t)sizeof(T));
+            if constexpr (W == 2) lines(P.b + t, cnt * (int64_t)sizeof(T));
+        } else {
+            lines(P.ein + t, cnt * (int64_t)sizeof(E));
         }
+    };
+    for (int64_t t0 = lo; t0 < hi; t0 += kTile) {
+        for (int q = lane; q < kRadix / 2; q += 32) reinterpret_cast<uint32_t*>(my_cnt)[q] = 0u;
+        __syncwarp();
+        const int64_t i0 = t0 + warp * (32 * ITEMS) + lane;
+        uint32_t key[ITEMS], rk[ITEMS / 2];  // ranks, two of 16 bits in a word
+        uint32_t okm = 0;
 #pragma unroll
-        for (int u = 0; u < kSortItems; ++u) {
+        for (int u = 0; u < ITEMS; ++u) {
+            key[u] = 0u;
+            if (i0 + u * 32 < hi && sort_key<I, T, W, FIRST>(P, i0 + u * 32, key[u])) okm |= 1u << u;
+        }
+        prefetch_tile(t0);
+#pragma unroll
+        for (int u = 0; u < ITEMS; ++u) {
+            const bool ok = (okm >> u) & 1u;
             const uint32_t d = (key[u] >> P.shift) & dmask;
             // the lanes holding the same digit: one ballot per digit bit
-            uint32_t peers = __ballot_sync(0xffffffffu, ok[u]);
-            for (int b = 0; b < P.bits; ++b) {
-                const uint32_t bal = __ballot_sync(0xffffffffu, (d >> b) & 1u);
-                peers &= ((d >> b) & 1u) ? bal : ~bal;
+            uint32_t peers = __ballot_sync(0xffffffffu, ok);
+#pragma unroll
+            for (int b = 0; b < kRadixBits; ++b) {
+                const uint32_t mine = (uint32_t)((int)(d << (31 - b)) >> 31);  // all ones or none
+                peers &= ~(__ballot_sync(0xffffffffu, mine != 0u) ^ mine);
             }
-            const uint32_t base = ok[u] ? s_cnt[warp][d] : 0u;
+            const uint32_t base = ok ? my_cnt[d] : 0u;
             __syncwarp();
-            if (ok[u] && (peers & lt) == 0u) s_cnt[warp][d] = base + __popc(peers);  // the lowest peer
+            if (ok && (peers & lt) == 0u) my_cnt[d] = (uint16_t)(base + __popc(peers));  // the lowest peer
             __syncwarp();
-            rk[u] = base + __popc(peers & lt);
+            const uint32_t r = base + __popc(peers & lt);
+            rk[u / 2] = (u & 1) ? (rk[u / 2] | (r << 16)) : r;
         }
         __syncthreads();
         // per digit: exclusive over the warps, then over the digits
@@ -249,8 +309,8 @@ __global__ void __launch_bounds__(kSortBlock) hg_scatter_kernel(SortPass<T> P) {
         if (threadIdx.x < R) {
 #pragma unroll
             for (int w = 0; w < kSortNW; ++w) {
-                const uint32_t c = s_cnt[w][threadIdx.x];
-                s_cnt[w][threadIdx.x] = tot;
+                const uint32_t c = s_cnt[w * kRadix + threadIdx.x];
+                s_cnt[w * kRadix + threadIdx.x] = (uint16_t)tot;
                 tot += c;
             }
         }
@@ -258,72 +318,87 @@ __global__ void __launch_bounds__(kSortBlock) hg_scatter_kernel(SortPass<T> P) {
         const uint32_t st = block_excl_u32(tot, s_w, &nvalid);
         if (threadIdx.x < R) s_start[threadIdx.x] = st;
         __syncthreads();
+        constexpr int B = ITEMS < 8 ? ITEMS : ITEMS / 2;  // values in flight per thread
+        static_assert(ITEMS % B == 0 && ITEMS % 2 == 0, "whole batches, ranks in pairs");
 #pragma unroll
-        for (int u = 0; u < kSortItems; ++u) {
-            const int64_t i = t0 + warp * (32 * kSortItems) + u * 32 + lane;
-            if (i >= hi) continue;
-            if (!ok[u]) {
-                P.dest[i] = kNoKey;
-                continue;
+        for (int h = 0; h < ITEMS; h += B) {
+            E e[B];
+#pragma unroll
+            for (int u = 0; u < B; ++u) {
+                const int64_t i = i0 + (h + u) * 32;
+                if (i >= hi) continue;
+                if constexpr (FIRST) {
+                    e[u] = make_elem<T, W>(__ldcs(P.a + i), W == 2 ? __ldcs(P.b + i) : T(0));
+                } else {
+                    e[u] = P.ein[i];
+                }
             }
-            const uint32_t d = (key[u] >> P.shift) & dmask;
-            const uint32_t within = s_cnt[warp][d] + rk[u];
-            const uint32_t lpos = s_start[d] + within;
-            P.dest[i] = s_off[d] + within;
-            s_key[lpos] = key[u];
-            s_a[lpos] = va[u];
-            if constexpr (W == 2) s_b[lpos] = vb[u];
+#pragma unroll
+            for (int u = 0; u < B; ++u) {
+                const int64_t i = i0 + (h + u) * 32;
+                if (i >= hi) continue;
+                const uint32_t k = key[h + u];
+                const uint32_t d = (k >> P.shift) & dmask;
+                const bool ok = (okm >> (h + u)) & 1u;
+                const uint32_t within = my_cnt[d] + ((rk[(h + u) / 2] >> (16 * ((h + u) & 1))) & 0xffffu);
+                if (ok) {
+                    const uint32_t lpos = s_start[d] + within;
+                    s_key[lpos] = k;
+                    s_e[lpos] = e[u];
+                }
+                if (P.dest) __stcs(P.dest + i, ok ? s_off[d] + within : kNoKey);
+            }
         }
         __syncthreads();
+#pragma unroll 4
         for (int q = threadIdx.x; q < (int)nvalid; q += kSortBlock) {
             const uint32_t k = s_key[q];
             const uint32_t d = (k >> P.shift) & dmask;
             const uint32_t pos = s_off[d] + (uint32_t)q - s_start[d];
             P.kout[pos] = k;
-            P.aout[pos] = s_a[q];
-            if constexpr (W == 2) P.bout[pos] = s_b[q];
+            P.eout[pos] = s_e[q];
         }
         __syncthreads();
         if (threadIdx.x < R) s_off[threadIdx.x] += tot;
     }
 }
 
-// Inverse of one pass: out[i] = in[dest[i]] over the pass's input order.
-// The first pass's inverse writes the caller's adjoints (0 or unchanged
-// for an element that left the sort, += with accumulation).
+// Inverse of one pass: out[i] = in[dest[i]] over the pass's input order, a block
+// taking kUnsortTile consecutive i at a time (their places lie in at most 256
+// runs, whose sectors stay in L1): 49 and 54 us for the two passes of 2^24 pairs,
+// 92 and 111 us with the pair in two arrays and a grid-wide stride.  The first pass's inverse writes the caller's
+// adjoints (0 or unchanged for an element that left the sort, += with
+// accumulation).
+constexpr int kUnsortTile = 8 * kSortBlock;
 template <class T, int W, bool FIRST>
 __global__ void __launch_bounds__(kSortBlock) hg_unsort_kernel(int64_t n, const uint32_t* nsorted,
-                                                               const uint32_t* dest, const T* ia, const T* ib,
-                                                               T* oa, T* ob, int accumulate) {
+                                                               const uint32_t* dest, const Elem<T, W>* in, T* oa,
+                                                               T* ob, Elem<T, W>* out, int accumulate) {
+    using E = Elem<T, W>;
+    constexpr int U = 8;
     const int64_t len = FIRST ? n : (int64_t)*nsorted;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x * 4;
-    for (int64_t i0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) * 4; i0 < len; i0 += stride) {
-        uint32_t d[4];
-        if (i0 + 4 <= len) {
-            const uint4 x = __ldcs(reinterpret_cast<const uint4*>(dest + i0));
-            d[0] = x.x; d[1] = x.y; d[2] = x.z; d[3] = x.w;
-        } else {
+    for (int64_t t0 = blockIdx.x * (int64_t)kUnsortTile; t0 < len; t0 += gridDim.x * (int64_t)kUnsortTile) {
+        const int64_t i0 = t0 + threadIdx.x;
+        uint32_t d[U];
+        E v[U];
 #pragma unroll
-            for (int j = 0; j < 4; ++j) d[j] = i0 + j < len ? dest[i0 + j] : kNoKey;
-        }
-        T va[4], vb[4];
+        for (int u = 0; u < U; ++u) d[u] = i0 + u * kSortBlock < len ? __ldcs(dest + i0 + u * kSortBlock) : kNoKey;
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            va[j] = d[j] != kNoKey ? ia[d[j]] : T(0);
-            vb[j] = (W == 2 && d[j] != kNoKey) ? ib[d[j]] : T(0);
-        }
+        for (int u = 0; u < U; ++u) v[u] = d[u] != kNoKey ? in[d[u]] : make_elem<T, W>(T(0), T(0));
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int64_t i = i0 + j;
-            if (i >= len) break;
-            if (FIRST && accumulate) {
-                if (d[j] != kNoKey) {
-                    oa[i] += va[j];
-                    if constexpr (W == 2) ob[i] += vb[j];
+        for (int u = 0; u < U; ++u) {
+            const int64_t i = i0 + u * kSortBlock;
+            if (i >= len) continue;
+            if constexpr (!FIRST) {
+                out[i] = v[u];
+            } else if (accumulate) {
+                if (d[u] != kNoKey) {
+                    oa[i] += v[u].a;
+                    if constexpr (W == 2) ob[i] += v[u].b;
                 }
             } else {
-                oa[i] = va[j];
-                if constexpr (W == 2) ob[i] = vb[j];
+                __stcs(oa + i, v[u].a);
+                if constexpr (W == 2) __stcs(ob + i, v[u].b);
             }
         }
     }
@@ -355,9 +430,8 @@ __device__ __forceinline__ SegS<Op> seg_rcomb(const SegS<Op>& e, const SegS<Op>&
 
 template <class Op, class T>
 struct SegArgs {
-    const uint32_t* keys;  // sorted bin numbers
-    const T* a;            // sorted values
-    const T* b;
+    const uint32_t* keys;              // sorted bin numbers
+    const Elem<T, Op::kWidth>* e;      // sorted values
     const uint32_t* nsorted;
     int64_t tiles;
     SegS<Op>* carry;       // [tiles] forward state before each tile
@@ -368,8 +442,7 @@ struct SegArgs {
     WsHeader* hdr;
     const T* hsbar_a;
     const T* hsbar_b;
-    T* oa;                 // [n] adjoints in sorted order
-    T* ob;
+    Elem<T, Op::kWidth>* o;  // [n] adjoints in sorted order
     T* hs_a;
     T* hs_b;
 };
@@ -384,72 +457,90 @@ __device__ __forceinline__ void ld_keys(const uint32_t* p, int64_t e, int64_t n,
     }
 }
 
-template <class T>
-__device__ __forceinline__ void ld_vals(const T* p, int64_t e, int64_t n, T pad, T (&o)[kSegV]) {
+// kSegV consecutive elements' values (pads past n), and their store
+template <class T, int W>
+__device__ __forceinline__ void ld_elems(const Elem<T, W>* p, int64_t e, int64_t n, T pad, T (&a)[kSegV],
+                                         T (&b)[kSegV]) {
     constexpr int VV = Vec16<T>::N;
     if (e + kSegV <= n) {
+        const T* q = reinterpret_cast<const T*>(p + e);
+        T f[W * kSegV];
 #pragma unroll
-        for (int q = 0; q < kSegV / VV; ++q) {
-            const Vec16<T> x = ld_vec_stream(p + e + q * VV);
+        for (int c = 0; c < W * kSegV / VV; ++c) {
+            const Vec16<T> x = ld_vec_stream(q + c * VV);
 #pragma unroll
-            for (int j = 0; j < VV; ++j) o[q * VV + j] = x.v[j];
+            for (int j = 0; j < VV; ++j) f[c * VV + j] = x.v[j];
+        }
+#pragma unroll
+        for (int j = 0; j < kSegV; ++j) {
+            a[j] = f[W * j];
+            b[j] = W == 2 ? f[W * j + (W - 1)] : T(0);
         }
     } else {
 #pragma unroll
-        for (int j = 0; j < kSegV; ++j) o[j] = e + j < n ? p[e + j] : pad;
+        for (int j = 0; j < kSegV; ++j) {
+            a[j] = e + j < n ? p[e + j].a : pad;
+            b[j] = e + j < n ? elem_b(p[e + j]) : T(0);
+        }
     }
 }
 
-template <class T>
-__device__ __forceinline__ void st_vals(T* p, int64_t e, int64_t n, const T (&v)[kSegV]) {
+template <class T, int W>
+__device__ __forceinline__ void st_elems(Elem<T, W>* p, int64_t e, int64_t n, const T (&a)[kSegV],
+                                         const T (&b)[kSegV]) {
     constexpr int VV = Vec16<T>::N;
     if (e + kSegV <= n) {
+        T* q = reinterpret_cast<T*>(p + e);
+        T f[W * kSegV];
 #pragma unroll
-        for (int q = 0; q < kSegV / VV; ++q) {
+        for (int j = 0; j < kSegV; ++j) {
+            f[W * j] = a[j];
+            if (W == 2) f[W * j + (W - 1)] = b[j];
+        }
+#pragma unroll
+        for (int c = 0; c < W * kSegV / VV; ++c) {
             Vec16<T> x;
 #pragma unroll
-            for (int j = 0; j < VV; ++j) x.v[j] = v[q * VV + j];
-            st_vec(p + e + q * VV, x);
+            for (int j = 0; j < VV; ++j) x.v[j] = f[c * VV + j];
+            st_vec(q + c * VV, x);
         }
     } else {
 #pragma unroll
         for (int j = 0; j < kSegV; ++j)
-            if (e + j < n) p[e + j] = v[j];
+            if (e + j < n) p[e + j] = make_elem<T, W>(a[j], b[j]);
     }
 }
 
 // Forward pass: each tile's forward segmented state before its first
-// element (the carry), by look-back.
-template <class Op, class T>
+// element (the carry), by look-back.  HS (the forward operator alone): the
+// states at the bins' last elements instead, into hs.
+template <class Op, class T, bool HS>
 __global__ void __launch_bounds__(kSegBlock) hg_seg_fwd_kernel(SegArgs<Op, T> A) {
     using S = SegS<Op>;
-    constexpr int NW = kSegBlock / 32, K = kSegK, V = kSegV;
+    constexpr int NW = kSegBlock / 32, K = kSegK, V = kSegV, W = Op::kWidth;
     __shared__ uint32_t s_tile;
     __shared__ S s_tot[K * NW];
+    __shared__ S s_carry;
     if (threadIdx.x == 0) s_tile = atomicAdd(&A.hdr->ticket[0], 1u);
     __syncthreads();
     const int64_t t = s_tile;
     const int64_t ns = (int64_t)*A.nsorted;
     const int64_t base = t * kSegTile;
+    uint32_t kk[K][V], kprev[K];
+    T av[K][V], bv[K][V];
     S agg[K];
 #pragma unroll
     for (int k = 0; k < K; ++k) {
         const int64_t e = base + (int64_t)k * kSegBlock * V + threadIdx.x * V;
-        uint32_t kk[V];
-        T av[V], bv[V];
-        ld_keys(A.keys, e, ns, kk);
-        ld_vals(A.a, e, ns, Op::pad_a(), av);
-        if constexpr (Op::kWidth == 2) ld_vals(A.b, e, ns, T(0), bv);
-        else {
-#pragma unroll
-            for (int j = 0; j < V; ++j) bv[j] = T(0);
-        }
-        uint32_t prev = (e > 0 && e - 1 < ns) ? A.keys[e - 1] : kNoKey;
+        ld_keys(A.keys, e, ns, kk[k]);
+        ld_elems<T, W>(A.e, e, ns, Op::pad_a(), av[k], bv[k]);
+        kprev[k] = (e > 0 && e - 1 < ns) ? A.keys[e - 1] : kNoKey;
+        uint32_t prev = kprev[k];
         S acc = seg_id<Op>();
 #pragma unroll
         for (int j = 0; j < V; ++j) {
-            if (e + j < ns) acc = seg_fcomb<Op>(acc, S{Op::pelem(av[j], bv[j]), kk[j] != prev ? 1u : 0u});
-            prev = kk[j];
+            if (e + j < ns) acc = seg_fcomb<Op>(acc, S{Op::pelem(av[k][j], bv[k][j]), kk[k][j] != prev ? 1u : 0u});
+            prev = kk[k][j];
         }
         agg[k] = acc;
     }
@@ -459,7 +550,32 @@ __global__ void __launch_bounds__(kSegBlock) hg_seg_fwd_kernel(SegArgs<Op, T> A)
     if ((threadIdx.x >> 5) == 0) {
         LookbackState<S> st{A.fA, A.fI};
         const S pre = lookback(t, st, total, seg_id<Op>(), fc, A.hdr);
-        if ((threadIdx.x & 31) == 0) A.carry[t] = pre;
+        if ((threadIdx.x & 31) == 0) {
+            if (HS) s_carry = pre;
+            else A.carry[t] = pre;
+        }
+    }
+    if constexpr (HS) {
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            const int64_t e = base + (int64_t)k * kSegBlock * V + threadIdx.x * V;
+            if (e >= ns) continue;
+            S lf = block_scan_excl<S, false, K, NW>(k, wex, s_tot, s_carry, fc);
+            const uint32_t knext = e + V < ns ? A.keys[e + V] : kNoKey;
+            uint32_t prev = kprev[k];
+#pragma unroll
+            for (int j = 0; j < V; ++j) {
+                const uint32_t key = kk[k][j];
+                lf = seg_fcomb<Op>(lf, S{Op::pelem(av[k][j], bv[k][j]), key != prev ? 1u : 0u});
+                prev = key;
+                const bool tail = e + j + 1 >= ns || (j + 1 < V ? kk[k][j + 1 < V ? j + 1 : j] : knext) != key;
+                if (e + j < ns && tail) {
+                    A.hs_a[key] = Op::out_a(lf.x);
+                    if constexpr (W == 2) A.hs_b[key] = Op::out_b(lf.x);
+                }
+            }
+        }
     }
 }
 
@@ -492,12 +608,7 @@ __global__ void __launch_bounds__(kSegBlock) hg_seg_bwd_kernel(SegArgs<Op, T> A)
     for (int k = 0; k < K; ++k) {
         const int64_t e = base + (int64_t)k * kSegBlock * V + threadIdx.x * V;
         ld_keys(A.keys, e, ns, kk[k]);
-        ld_vals(A.a, e, ns, Op::pad_a(), av[k]);
-        if constexpr (W == 2) ld_vals(A.b, e, ns, T(0), bv[k]);
-        else {
-#pragma unroll
-            for (int j = 0; j < V; ++j) bv[k][j] = T(0);
-        }
+        ld_elems<T, W>(A.e, e, ns, Op::pad_a(), av[k], bv[k]);
         kprev[k] = (e > 0 && e - 1 < ns) ? A.keys[e - 1] : kNoKey;
         knext[k] = (e + V < ns) ? A.keys[e + V] : kNoKey;
         S f = seg_id<Op>();
@@ -566,8 +677,7 @@ __global__ void __launch_bounds__(kSegBlock) hg_seg_bwd_kernel(SegArgs<Op, T> A)
             }
             rr = seg_rcomb<Op>(rr, S{Op::pelem(av[k][j], bv[k][j]), tail ? 1u : 0u});
         }
-        st_vals(A.oa, e, ns, oa);
-        if constexpr (W == 2) st_vals(A.ob, e, ns, ob);
+        st_elems<T, W>(A.o, e, ns, oa, ob);
     }
 }
 
@@ -584,7 +694,7 @@ __global__ void hg_fill_kernel(int64_t m, T* hs_a, T* hs_b) {
 constexpr int kMaxPasses = 4;  // 31 key bits in passes of at most 8
 
 struct HgLayout {
-    size_t off_cnt, off_rowtot, off_k[2], off_a[2], off_b[2], off_dest[kMaxPasses], off_carry, off_slots;
+    size_t off_cnt, off_rowtot, off_k[2], off_e[2], off_dest[kMaxPasses], off_carry, off_slots;
     size_t slot_bytes, total;
     int64_t tiles;
 };
@@ -610,8 +720,7 @@ HgLayout hg_layout(int64_t n, int64_t m) {
     L.off_rowtot = take(sizeof(uint32_t) * kRadix);
     for (int q = 0; q < 2; ++q) {
         L.off_k[q] = take(sizeof(uint32_t) * nn);
-        L.off_a[q] = take(sizeof(T) * nn);
-        L.off_b[q] = Op::kWidth == 2 ? take(sizeof(T) * nn) : L.off_a[q];
+        L.off_e[q] = take(sizeof(Elem<T, Op::kWidth>) * nn);
     }
     const int passes = (key_bits(m) + kRadixBits - 1) / kRadixBits;
     for (int p = 0; p < passes; ++p) L.off_dest[p] = take(sizeof(uint32_t) * nn);
@@ -631,12 +740,53 @@ int sms_now() {
     return sms > 0 ? sms : 1;
 }
 
+// the sort's passes with tiles of ITEMS elements per thread; the sorted data end
+// up in buffer (passes & 1)
+template <class T, int W, class I, int ITEMS>
+int run_sort(SortPass<T, W> SP, char* w, const size_t (&off_k)[2], const size_t (&off_e)[2], const size_t* off_dest,
+             bool keep_dest, uint32_t* nsorted, int passes, int bits, cudaStream_t s) {
+    constexpr int kTile = kSortBlock * ITEMS;
+    constexpr size_t smem = sort_smem<T, W, ITEMS>();
+    auto first = hg_scatter_kernel<I, T, W, true, ITEMS>;
+    auto later = hg_scatter_kernel<I, T, W, false, ITEMS>;
+    if (cudaFuncSetAttribute(first, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+        cudaFuncSetAttribute(later, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+        return ADPAR_ERR_CUDA;
+    const int dbits = (bits + passes - 1) / passes;
+    // one wave of the scatter kernel (two blocks per SM): every block's chunk is in flight at once
+    const int G = (int)std::max<int64_t>(
+        1, std::min<int64_t>({(SP.n + kTile - 1) / kTile, (int64_t)kSortMaxGrid, (int64_t)sms_now() * 2}));
+    SP.G = G;
+    for (int p = 0; p < passes; ++p) {
+        const int src = p & 1, dst = (p + 1) & 1;
+        SP.shift = p * dbits;
+        SP.bits = std::min(dbits, bits - p * dbits);
+        SP.kin = reinterpret_cast<const uint32_t*>(w + off_k[src]);
+        SP.ein = reinterpret_cast<const Elem<T, W>*>(w + off_e[src]);
+        SP.kout = reinterpret_cast<uint32_t*>(w + off_k[dst]);
+        SP.eout = reinterpret_cast<Elem<T, W>*>(w + off_e[dst]);
+        SP.dest = keep_dest ? reinterpret_cast<uint32_t*>(w + off_dest[p]) : nullptr;
+        if (p == 0) {
+            hg_count_kernel<I, T, W, true><<<G, kSortBlock, 0, s>>>(SP, kTile);
+            hg_scan_counts_kernel<<<1 << SP.bits, kSortBlock, 0, s>>>(SP.cnt, SP.rowtot, G, nsorted);
+            first<<<G, kSortBlock, smem, s>>>(SP);
+        } else {
+            hg_count_kernel<I, T, W, false><<<G, kSortBlock, 0, s>>>(SP, kTile);
+            hg_scan_counts_kernel<<<1 << SP.bits, kSortBlock, 0, s>>>(SP.cnt, SP.rowtot, G, nullptr);
+            later<<<G, kSortBlock, smem, s>>>(SP);
+        }
+    }
+    return ADPAR_OK;
+}
+
+// abar NULL: the forward operator alone (hs_a given)
 template <class Op, class T, class I>
 int run_hist_general(int64_t n, int64_t m, const void* a, const void* b, const void* inds, const void* hsbar_a,
                      const void* hsbar_b, void* abar, void* bbar, void* hs_a, void* hs_b, uint32_t flags,
                      void* work, size_t work_bytes, cudaStream_t s) {
     using S = SegS<Op>;
     constexpr int W = Op::kWidth;
+    using E = Elem<T, W>;
     const HgLayout L = hg_layout<Op, T>(n, m);
     if (work == nullptr || work_bytes < L.total || (reinterpret_cast<uintptr_t>(work) & 255u))
         return ADPAR_ERR_WORKSPACE;
@@ -653,45 +803,22 @@ int run_hist_general(int64_t n, int64_t m, const void* a, const void* b, const v
     // key bits: bin numbers are below m (out-of-range elements leave in pass 0)
     const int bits = key_bits(m);
     const int passes = (bits + kRadixBits - 1) / kRadixBits;
-    const int dbits = (bits + passes - 1) / passes;
-    // one wave of the scatter kernel: every block's chunk is in flight at once
-    const int sms = sms_now();
-    int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, hg_scatter_kernel<I, T, W, false>, kSortBlock, 0) !=
-            cudaSuccess || per_sm < 1)
-        per_sm = 1;
-    const int G = (int)std::max<int64_t>(
-        1, std::min<int64_t>({(n + kChunkAlign - 1) / kChunkAlign, (int64_t)kSortMaxGrid, (int64_t)sms * per_sm}));
     uint32_t* nsorted = &hdr->done[0];
-    SortPass<T> SP{};
+    SortPass<T, W> SP{};
     SP.n = n;
     SP.m = m;
     SP.inds = inds;
+    SP.a = static_cast<const T*>(a);
+    SP.b = static_cast<const T*>(b);
     SP.cnt = reinterpret_cast<uint32_t*>(w + L.off_cnt);
     SP.rowtot = reinterpret_cast<uint32_t*>(w + L.off_rowtot);
     SP.nsorted = nsorted;
-    SP.G = G;
-    for (int p = 0; p < passes; ++p) {
-        const int src = p & 1, dst = (p + 1) & 1;
-        SP.shift = p * dbits;
-        SP.bits = std::min(dbits, bits - p * dbits);
-        SP.kin = reinterpret_cast<const uint32_t*>(w + L.off_k[src]);
-        SP.ain = p == 0 ? static_cast<const T*>(a) : reinterpret_cast<const T*>(w + L.off_a[src]);
-        SP.bin = p == 0 ? static_cast<const T*>(b) : reinterpret_cast<const T*>(w + L.off_b[src]);
-        SP.kout = reinterpret_cast<uint32_t*>(w + L.off_k[dst]);
-        SP.aout = reinterpret_cast<T*>(w + L.off_a[dst]);
-        SP.bout = reinterpret_cast<T*>(w + L.off_b[dst]);
-        SP.dest = reinterpret_cast<uint32_t*>(w + L.off_dest[p]);
-        if (p == 0) {
-            hg_count_kernel<I, T, true><<<G, kSortBlock, 0, s>>>(SP);
-            hg_scan_counts_kernel<<<1 << SP.bits, kSortBlock, 0, s>>>(SP.cnt, SP.rowtot, G, nsorted);
-            hg_scatter_kernel<I, T, W, true><<<G, kSortBlock, 0, s>>>(SP);
-        } else {
-            hg_count_kernel<I, T, false><<<G, kSortBlock, 0, s>>>(SP);
-            hg_scan_counts_kernel<<<1 << SP.bits, kSortBlock, 0, s>>>(SP.cnt, SP.rowtot, G, nullptr);
-            hg_scatter_kernel<I, T, W, false><<<G, kSortBlock, 0, s>>>(SP);
-        }
-    }
+    const bool vjp = abar != nullptr;
+    const int st = n >= kBigSort ? run_sort<T, W, I, big_items<T, W>()>(SP, w, L.off_k, L.off_e, L.off_dest, vjp,
+                                                                        nsorted, passes, bits, s)
+                                 : run_sort<T, W, I, kSmallItems>(SP, w, L.off_k, L.off_e, L.off_dest, vjp, nsorted,
+                                                                  passes, bits, s);
+    if (st != ADPAR_OK) return st;
     // the sorted data sit in buffer fin; the other buffer takes the
     // sorted-order adjoints, and the inverse passes alternate between them
     const int fin = passes & 1;
@@ -699,8 +826,7 @@ int run_hist_general(int64_t n, int64_t m, const void* a, const void* b, const v
     unsigned long long* slots = reinterpret_cast<unsigned long long*>(w + L.off_slots);
     SegArgs<Op, T> A{};
     A.keys = reinterpret_cast<const uint32_t*>(w + L.off_k[fin]);
-    A.a = reinterpret_cast<const T*>(w + L.off_a[fin]);
-    A.b = reinterpret_cast<const T*>(w + L.off_b[fin]);
+    A.e = reinterpret_cast<const E*>(w + L.off_e[fin]);
     A.nsorted = nsorted;
     A.tiles = L.tiles;
     A.carry = reinterpret_cast<S*>(w + L.off_carry);
@@ -711,27 +837,28 @@ int run_hist_general(int64_t n, int64_t m, const void* a, const void* b, const v
     A.hdr = hdr;
     A.hsbar_a = static_cast<const T*>(hsbar_a);
     A.hsbar_b = static_cast<const T*>(hsbar_b);
-    A.oa = reinterpret_cast<T*>(w + L.off_a[1 - fin]);
-    A.ob = reinterpret_cast<T*>(w + L.off_b[1 - fin]);
+    A.o = reinterpret_cast<E*>(w + L.off_e[1 - fin]);
     A.hs_a = static_cast<T*>(hs_a);
     A.hs_b = static_cast<T*>(hs_b);
-    hg_seg_fwd_kernel<Op, T><<<(unsigned)L.tiles, kSegBlock, 0, s>>>(A);
+    if (!vjp) {
+        hg_seg_fwd_kernel<Op, T, true><<<(unsigned)L.tiles, kSegBlock, 0, s>>>(A);
+        return cudaGetLastError() == cudaSuccess ? ADPAR_OK : ADPAR_ERR_CUDA;
+    }
+    hg_seg_fwd_kernel<Op, T, false><<<(unsigned)L.tiles, kSegBlock, 0, s>>>(A);
     hg_seg_bwd_kernel<Op, T><<<(unsigned)L.tiles, kSegBlock, 0, s>>>(A);
     const int acc = (flags & ADPAR_ACCUMULATE) ? 1 : 0;
-    const int ublocks = (int)std::max<int64_t>(1, std::min<int64_t>((n / 4 + kSortBlock) / kSortBlock,
-                                                                       (int64_t)sms * 8));
+    const int ublocks =
+        (int)std::max<int64_t>(1, std::min<int64_t>((n + kUnsortTile - 1) / kUnsortTile, (int64_t)sms_now() * 16));
     int cur = 1 - fin;
     for (int p = passes - 1; p >= 0; --p) {
         const uint32_t* dest = reinterpret_cast<const uint32_t*>(w + L.off_dest[p]);
-        const T* ia = reinterpret_cast<const T*>(w + L.off_a[cur]);
-        const T* ib = reinterpret_cast<const T*>(w + L.off_b[cur]);
+        const E* in = reinterpret_cast<const E*>(w + L.off_e[cur]);
         if (p == 0) {
-            hg_unsort_kernel<T, W, true><<<ublocks, kSortBlock, 0, s>>>(n, nsorted, dest, ia, ib, static_cast<T*>(abar),
-                                                                       static_cast<T*>(bbar), acc);
+            hg_unsort_kernel<T, W, true><<<ublocks, kSortBlock, 0, s>>>(n, nsorted, dest, in, static_cast<T*>(abar),
+                                                                       static_cast<T*>(bbar), nullptr, acc);
         } else {
-            T* oa = reinterpret_cast<T*>(w + L.off_a[1 - cur]);
-            T* ob = reinterpret_cast<T*>(w + L.off_b[1 - cur]);
-            hg_unsort_kernel<T, W, false><<<ublocks, kSortBlock, 0, s>>>(n, nsorted, dest, ia, ib, oa, ob, acc);
+            hg_unsort_kernel<T, W, false><<<ublocks, kSortBlock, 0, s>>>(
+                n, nsorted, dest, in, nullptr, nullptr, reinterpret_cast<E*>(w + L.off_e[1 - cur]), acc);
             cur = 1 - cur;
         }
     }
@@ -781,11 +908,11 @@ size_t hist_general_workspace_size(adpar_opdesc d, int64_t n, int64_t m) {
 
 }  // namespace adpar
 
-extern "C" int adpar_vjp_hist_general(adpar_opdesc d, int64_t n, int64_t m, const void* a, const void* b,
-                                      const void* inds, int itype, const void* hsbar_a, const void* hsbar_b,
-                                      void* abar, void* bbar, void* hs_a, void* hs_b, uint32_t flags, void* work,
-                                      size_t work_bytes, void* stream) {
-    using namespace adpar;
+namespace adpar {
+namespace {
+int hist_general_impl(adpar_opdesc d, int64_t n, int64_t m, const void* a, const void* b, const void* inds, int itype,
+                      const void* hsbar_a, const void* hsbar_b, void* abar, void* bbar, void* hs_a, void* hs_b,
+                      uint32_t flags, void* work, size_t work_bytes, void* stream, bool primal_only) {
     if (n < 0 || m < 0) return ADPAR_ERR_INVALID;
     if (d.op < ADPAR_OP_ADD || d.op > ADPAR_OP_LINREC) return ADPAR_ERR_INVALID;
     if (d.dtype != ADPAR_F32 && d.dtype != ADPAR_F64) return ADPAR_ERR_INVALID;
@@ -797,7 +924,10 @@ extern "C" int adpar_vjp_hist_general(adpar_opdesc d, int64_t n, int64_t m, cons
     if (n >= (int64_t)0xffffffffu || m > ((int64_t)1 << 31)) return ADPAR_ERR_UNSUPPORTED;
     if (want_w == 2 && hs_a && !hs_b) return ADPAR_ERR_INVALID;
     if (hs_a == nullptr && hs_b != nullptr) return ADPAR_ERR_INVALID;
-    if (n > 0) {
+    if (primal_only) {
+        if ((m > 0 && (!hs_a || (want_w == 2 && !hs_b))) || (n > 0 && (!a || !inds || (want_w == 2 && !b))))
+            return ADPAR_ERR_INVALID;
+    } else if (n > 0) {
         if (!a || !inds || !abar || (m > 0 && !hsbar_a)) return ADPAR_ERR_INVALID;
         if (want_w == 2 && (!b || !bbar || (m > 0 && !hsbar_b))) return ADPAR_ERR_INVALID;
     }
@@ -814,4 +944,20 @@ extern "C" int adpar_vjp_hist_general(adpar_opdesc d, int64_t n, int64_t m, cons
                                                       hs_b, flags, work, work_bytes, s);
     return dispatch_hist_general<double, int64_t>(d.op, n, m, a, b, inds, hsbar_a, hsbar_b, abar, bbar, hs_a, hs_b,
                                                   flags, work, work_bytes, s);
+}
+}  // namespace
+}  // namespace adpar
+
+extern "C" int adpar_vjp_hist_general(adpar_opdesc d, int64_t n, int64_t m, const void* a, const void* b,
+                                      const void* inds, int itype, const void* hsbar_a, const void* hsbar_b,
+                                      void* abar, void* bbar, void* hs_a, void* hs_b, uint32_t flags, void* work,
+                                      size_t work_bytes, void* stream) {
+    return adpar::hist_general_impl(d, n, m, a, b, inds, itype, hsbar_a, hsbar_b, abar, bbar, hs_a, hs_b, flags, work,
+                                    work_bytes, stream, false);
+}
+
+extern "C" int adpar_hist_general(adpar_opdesc d, int64_t n, int64_t m, const void* a, const void* b, const void* inds,
+                                  int itype, void* hs_a, void* hs_b, void* work, size_t work_bytes, void* stream) {
+    return adpar::hist_general_impl(d, n, m, a, b, inds, itype, nullptr, nullptr, nullptr, nullptr, hs_a, hs_b, 0u,
+                                    work, work_bytes, stream, true);
 }
