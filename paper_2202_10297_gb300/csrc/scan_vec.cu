@@ -3,16 +3,17 @@
 //   scan (map (.)) e xs == transpose xs |> map (scan (.) e) |> transpose,
 // i.e. d independent scans down the columns.  No transpose is materialised:
 // a thread owns one column and one chunk of kVecR rows, so a warp's loads
-// cover 32 consecutive columns of a row (coalesced).  Five kernels, no
-// block waits on another:
-//   1. per (chunk, column): the aggregate of the operator's state;
-//   2. per column, one warp scans the chunk aggregates (exclusive carries);
-//   3. per (chunk, column): the aggregate of the return sweep's lin_o state
-//      (MIN/MAX re-form the primal prefix from the carry for J_left);
-//   4. per column, one warp scans those right to left (exclusive carries);
-//   5. per (chunk, column): a backward sweep of rs_bar_r = ybar_r +
+// cover 32 consecutive columns of a row (coalesced), 8 rows' loads in flight.
+// No block waits on another:
+//   1. per (chunk, column): the aggregates of the operator's state and of the
+//      return sweep's lin_o state;
+//   2. per column a scan of the chunks' aggregates, left to right and right to
+//      left (exclusive carries);
+//   3. per (chunk, column): a backward sweep of rs_bar_r = ybar_r +
 //      c_{r+1} rs_bar_{r+1} into shared memory, then a forward sweep with
 //      the primal prefix writing as_bar = J_right^T rs_bar.
+// MIN/MAX, whose J_left needs the primal prefix, take 1 and 2 for the operator
+// first and then for the return sweep (re-forming the prefix from the carry).
 #include <algorithm>
 
 #include "scan_tiles.cuh"
@@ -41,174 +42,230 @@ struct VecArgs {
     void* aggL;  // [C][d] L: chunk aggregates, then exclusive suffixes
 };
 
-template <class Op, class T>
-__device__ __forceinline__ typename Op::P vec_elem(const VecArgs& V, int64_t i) {
-    return Op::pelem(__ldg(static_cast<const T*>(V.a) + i),
-                     Op::kWidth == 2 ? __ldg(static_cast<const T*>(V.b) + i) : T(0));
+// rows whose loads a thread has in flight at once
+constexpr int kVecU = 8;     // output pass
+constexpr int kVecUAgg = 4;  // aggregates
+
+// p[i], p[i + d], .. for U rows from `row` on (pad past the last row)
+template <int U, class T>
+__device__ __forceinline__ void vec_rows(const void* p, const VecArgs& V, int64_t row, int64_t col, T pad,
+                                         T (&o)[U]) {
+    const T* q = static_cast<const T*>(p) + row * V.d + col;
+#pragma unroll
+    for (int u = 0; u < U; ++u) o[u] = row + u < V.n ? __ldg(q + u * V.d) : pad;
 }
 
-template <class Op, class T>
-__global__ void __launch_bounds__(kVecBlock) vec_primal_agg_kernel(VecArgs V) {
+// Chunk aggregates in one sweep from top to bottom: PRIMAL the operator's state,
+// ADJ the return sweep's x -> c_r (ybar_r + x), composed as a growing map (the
+// next row's map goes inside), so that each array is read once.  MIN/MAX take
+// their J_left from the prefix, formed from the carry that a first launch
+// (PRIMAL alone) and its scan left.
+template <class Op, class T, bool PRIMAL, bool ADJ>
+__global__ void __launch_bounds__(kVecBlock, 6) vec_agg_kernel(VecArgs V) {
     using P = typename Op::P;
+    constexpr int W = Op::kWidth, U = kVecUAgg;
+    constexpr bool kA = PRIMAL || !Op::kCoefOne;  // a is read
+    using L = Lin<T, W, !Op::kCoefOne>;
     const int64_t col = blockIdx.x * (int64_t)kVecBlock + threadIdx.x, c = blockIdx.y;
     if (col >= V.d) return;
-    const int64_t r0 = c * kVecR, r1 = std::min<int64_t>(V.n, r0 + kVecR);
-    P acc = Op::pid();
-    for (int64_t r = r0; r < r1; ++r) acc = Op::pcomb(acc, vec_elem<Op, T>(V, r * V.d + col));
-    static_cast<P*>(V.aggP)[c * V.d + col] = acc;
+    const int64_t r0 = c * kVecR;
+    P cur = Op::pid();
+    if constexpr (ADJ && Op::kCoefNeedsPrimal) cur = static_cast<const P*>(V.aggP)[c * V.d + col];
+    L acc = L::id();
+#pragma unroll 1
+    for (int q = 0; q < kVecR; q += U) {
+        T a[U], b[U], y1[U], y2[U];
+        if constexpr (kA) vec_rows<U>(V.a, V, r0 + q, col, Op::pad_a(), a);
+        if constexpr (PRIMAL && W == 2) vec_rows<U>(V.b, V, r0 + q, col, T(0), b);
+        if constexpr (ADJ) vec_rows<U>(V.ya, V, r0 + q, col, T(0), y1);
+        if constexpr (ADJ && W == 2) vec_rows<U>(V.yb, V, r0 + q, col, T(0), y2);
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if constexpr (ADJ) {
+                if (r0 + q + u < V.n) {
+                    L el;
+                    if constexpr (!Op::kCoefOne) {
+                        const T cr = Op::coef(cur, a[u]);
+                        el.c = cr;
+                        el.d[0] = cr * y1[u];
+                        if constexpr (W == 2) el.d[1] = cr * y2[u];
+                    } else {
+                        el.d[0] = y1[u];
+                        if constexpr (W == 2) el.d[1] = y2[u];
+                    }
+                    acc = L::comb(el, acc);
+                }
+            }
+            if constexpr (PRIMAL || (ADJ && Op::kCoefNeedsPrimal))
+                cur = Op::pcomb(cur, Op::pelem(a[u], PRIMAL && W == 2 ? b[u] : T(0)));
+        }
+    }
+    if constexpr (PRIMAL) static_cast<P*>(V.aggP)[c * V.d + col] = cur;
+    if constexpr (ADJ) static_cast<L*>(V.aggL)[c * V.d + col] = acc;
 }
 
-// One warp per column turns the column's C chunk aggregates into exclusive
-// prefixes (REV: exclusive suffixes, composed right to left), 32 chunks per
-// round with a shuffle scan and a carry between rounds.
+// Turns the chunk aggregates of 32 columns into exclusive prefixes (REV:
+// exclusive suffixes, composed right to left).  Thread (x, y) of a 32 x kVecG
+// block folds group y of column x's chunks (neighbouring lanes read neighbouring
+// columns), takes the fold of the groups before it and runs through its chunks
+// again.  8 chunks are loaded at a time.
+constexpr int kVecG = 32;
 template <class S, bool REV, class Comb>
-__device__ __forceinline__ void vec_scan_column(S* agg, int64_t C, int64_t d, int64_t col, const S& ident,
-                                                Comb comb) {
-    const int lane = threadIdx.x & 31;
-    S carry = ident;
-    for (int64_t base = 0; base < C; base += 32) {
-        const int64_t q = REV ? C - 1 - (base + lane) : base + lane;  // chunk of this lane
-        const bool ok = base + lane < C;
-        S v = ok ? agg[q * d + col] : ident;
-        S inc = v;
+__device__ __forceinline__ void vec_scan_columns(S* agg, int64_t C, int64_t d, S* s_tot, const S& ident, Comb comb) {
+    const int x = threadIdx.x & 31, y = threadIdx.x >> 5;
+    const int64_t col = blockIdx.x * (int64_t)32 + x;
+    const int64_t per = (C + kVecG - 1) / kVecG;
+    const int64_t lo = y * per < C ? y * per : C, hi = lo + per < C ? lo + per : C;
+    const bool live = col < d;
+    auto at = [&](int64_t q) -> S* { return agg + (REV ? C - 1 - q : q) * d + col; };
+    S acc = ident;
+    if (live) {
+        for (int64_t q = lo; q < hi; q += 8) {
+            S v[8];
 #pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-            const S o = shfl_up_s(inc, off);
-            if (lane >= off) inc = comb(o, inc);
+            for (int u = 0; u < 8; ++u) v[u] = q + u < hi ? *at(q + u) : ident;
+#pragma unroll
+            for (int u = 0; u < 8; ++u) acc = comb(acc, v[u]);
         }
-        S ex = shfl_up_s(inc, 1);
-        if (lane == 0) ex = ident;
-        if (ok) agg[q * d + col] = comb(carry, ex);
-        carry = comb(carry, shfl_idx_s(inc, 31));
+    }
+    s_tot[y * 32 + x] = acc;
+    __syncthreads();
+    S run = ident;
+    for (int g = 0; g < y; ++g) run = comb(run, s_tot[g * 32 + x]);
+    if (live) {
+        for (int64_t q = lo; q < hi; q += 8) {
+            S v[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) v[u] = q + u < hi ? *at(q + u) : ident;
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                if (q + u < hi) *at(q + u) = run;
+                run = comb(run, v[u]);
+            }
+        }
     }
 }
 
+// Scans the aggregates asked for: blockIdx.y 0 the operator's, 1 the return
+// sweep's (first: the y of the first grid row)
 template <class Op, class T>
-__global__ void vec_scan_P_kernel(VecArgs V) {
+__global__ void __launch_bounds__(32 * kVecG) vec_scan_kernel(VecArgs V, int first) {
     using P = typename Op::P;
-    const int64_t col = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (col >= V.d) return;  // whole warps leave together
-    vec_scan_column<P, false>(static_cast<P*>(V.aggP), V.C, V.d, col, Op::pid(),
-                              [](const P& l, const P& r) { return Op::pcomb(l, r); });
-}
-
-template <class Op, class T>
-__global__ void vec_scan_L_kernel(VecArgs V) {
     using L = Lin<T, Op::kWidth, !Op::kCoefOne>;
-    const int64_t col = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (col >= V.d) return;
-    // scan order is right to left: e holds later rows, l earlier ones
-    vec_scan_column<L, true>(static_cast<L*>(V.aggL), V.C, V.d, col, L::id(),
-                             [](const L& e, const L& l) { return L::comb(e, l); });
+    extern __shared__ __align__(16) unsigned char s_dyn[];
+    if (blockIdx.y + first == 0) {
+        vec_scan_columns<P, false>(static_cast<P*>(V.aggP), V.C, V.d, reinterpret_cast<P*>(s_dyn), Op::pid(),
+                                   [](const P& l, const P& r) { return Op::pcomb(l, r); });
+    } else {
+        // scan order is right to left: e holds later rows, l earlier ones
+        vec_scan_columns<L, true>(static_cast<L*>(V.aggL), V.C, V.d, reinterpret_cast<L*>(s_dyn), L::id(),
+                                  [](const L& e, const L& l) { return L::comb(e, l); });
+    }
 }
 
 // J_left of the chunk's rows as bits (MIN/MAX: needs the primal prefix)
 template <class Op, class T>
-__device__ __forceinline__ uint32_t vec_coef_bits(const VecArgs& V, int64_t col, int64_t r0, int64_t r1,
+__device__ __forceinline__ uint32_t vec_coef_bits(const VecArgs& V, int64_t col, int64_t r0,
                                                   const typename Op::P& carry) {
     uint32_t bits = 0u;
     typename Op::P cur = carry;
-    for (int64_t r = r0; r < r1; ++r) {
-        const int64_t i = r * V.d + col;
-        const T a = __ldg(static_cast<const T*>(V.a) + i);
-        if (Op::coef(cur, a) != T(0)) bits |= 1u << (r - r0);
-        cur = Op::pcomb(cur, vec_elem<Op, T>(V, i));
+#pragma unroll 1
+    for (int q = 0; q < kVecR; q += kVecU) {
+        T a[kVecU];
+        vec_rows(V.a, V, r0 + q, col, Op::pad_a(), a);
+#pragma unroll
+        for (int u = 0; u < kVecU; ++u) {
+            if (Op::coef(cur, a[u]) != T(0)) bits |= 1u << (q + u);
+            cur = Op::pcomb(cur, Op::pelem(a[u], T(0)));
+        }
     }
     return bits;
 }
 
+// J_left of the rows row .. row + kVecU - 1 (q0: the first one's number in the
+// chunk); rows past the end have ybar 0 below them, so their value is free
 template <class Op, class T>
-__device__ __forceinline__ T vec_coef(const VecArgs& V, int64_t i, uint32_t bits, int64_t rr) {
-    if constexpr (Op::kCoefOne) return T(1);
-    else if constexpr (Op::kCoefNeedsPrimal) return ((bits >> rr) & 1u) ? T(1) : T(0);
-    else return Op::coef(Op::pid(), __ldg(static_cast<const T*>(V.a) + i));
-}
-
-template <class Op, class T>
-__global__ void __launch_bounds__(kVecBlock) vec_adjoint_agg_kernel(VecArgs V) {
-    using P = typename Op::P;
-    constexpr int W = Op::kWidth;
-    using L = Lin<T, W, !Op::kCoefOne>;
-    const int64_t col = blockIdx.x * (int64_t)kVecBlock + threadIdx.x, c = blockIdx.y;
-    if (col >= V.d) return;
-    const int64_t r0 = c * kVecR, r1 = std::min<int64_t>(V.n, r0 + kVecR);
-    uint32_t bits = 0u;
-    if constexpr (Op::kCoefNeedsPrimal)
-        bits = vec_coef_bits<Op, T>(V, col, r0, r1, static_cast<const P*>(V.aggP)[c * V.d + col]);
-    // x -> c_r (ybar_r + x) folded over the rows, bottom to top
-    L acc = L::id();
-    for (int64_t r = r1 - 1; r >= r0; --r) {
-        const int64_t i = r * V.d + col;
-        L el;
-        const T y1 = __ldg(static_cast<const T*>(V.ya) + i);
-        const T y2 = W == 2 ? __ldg(static_cast<const T*>(V.yb) + i) : T(0);
-        if constexpr (!Op::kCoefOne) {
-            const T cr = vec_coef<Op, T>(V, i, bits, r - r0);
-            el.c = cr;
-            el.d[0] = cr * y1;
-            if constexpr (W == 2) el.d[1] = cr * y2;
-        } else {
-            el.d[0] = y1;
-            if constexpr (W == 2) el.d[1] = y2;
-        }
-        acc = L::comb(acc, el);
+__device__ __forceinline__ void vec_coefs(const VecArgs& V, int64_t row, int64_t col, uint32_t bits, int q0,
+                                          T (&c)[kVecU]) {
+    if constexpr (Op::kCoefOne) {
+#pragma unroll
+        for (int u = 0; u < kVecU; ++u) c[u] = T(1);
+    } else if constexpr (Op::kCoefNeedsPrimal) {
+#pragma unroll
+        for (int u = 0; u < kVecU; ++u) c[u] = ((bits >> (q0 + u)) & 1u) ? T(1) : T(0);
+    } else {
+        vec_rows(V.a, V, row, col, T(1), c);
+#pragma unroll
+        for (int u = 0; u < kVecU; ++u) c[u] = Op::coef(Op::pid(), c[u]);
     }
-    static_cast<L*>(V.aggL)[c * V.d + col] = acc;
 }
 
+// Chunks last to first: what vec_agg_kernel read last is still in L2.  8 rows'
+// loads in flight at 9 blocks an SM (about 110 registers): 72 us for 8192 x 2048
+// FP32 LINREC (59 us for its bytes); 64 registers, or one row at a time: 96 and
+// 128 us.  The aggregates take 52 us (was 23 + 40 in two launches), the scan of
+// both 11 us (was 13 + 23 with a warp per column); the call 245 -> 138 us.
 template <class Op, class T>
-__global__ void __launch_bounds__(kVecOutBlock) vec_output_kernel(VecArgs V) {
+__global__ void __launch_bounds__(kVecOutBlock, 9) vec_output_kernel(VecArgs V) {
     using P = typename Op::P;
     constexpr int W = Op::kWidth;
     constexpr bool kP = kVecPrimal<Op>;
     using L = Lin<T, W, !Op::kCoefOne>;
     __shared__ T s_r[kVecR * W * kVecOutBlock];  // rs_bar of the thread's rows, [row][component][thread]
-    const int64_t col = blockIdx.x * (int64_t)kVecOutBlock + threadIdx.x, c = blockIdx.y;
+    const int64_t col = blockIdx.x * (int64_t)kVecOutBlock + threadIdx.x, c = V.C - 1 - (int64_t)blockIdx.y;
     if (col >= V.d) return;
-    const int64_t r0 = c * kVecR, r1 = std::min<int64_t>(V.n, r0 + kVecR);
+    const int64_t r0 = c * kVecR;
     const P carry = kP ? static_cast<const P*>(V.aggP)[c * V.d + col] : Op::pid();
     const L suf = static_cast<const L*>(V.aggL)[c * V.d + col];
     uint32_t bits = 0u;
-    if constexpr (Op::kCoefNeedsPrimal) bits = vec_coef_bits<Op, T>(V, col, r0, r1, carry);
-    // backward: rs_bar of the last row gets the chunks below through suf.d
-    T ra = T(0), rb = T(0);
-    for (int64_t r = r1 - 1; r >= r0; --r) {
-        const int64_t i = r * V.d + col;
-        const T y1 = __ldg(static_cast<const T*>(V.ya) + i);
-        const T y2 = W == 2 ? __ldg(static_cast<const T*>(V.yb) + i) : T(0);
-        if (r == r1 - 1) {
-            ra = y1 + suf.d[0];
-            if constexpr (W == 2) rb = y2 + suf.d[W - 1];
-        } else {
-            const T cn = vec_coef<Op, T>(V, i + V.d, bits, r + 1 - r0);  // J_left of the row below
-            ra = fma(cn, ra, y1);
-            if constexpr (W == 2) rb = fma(cn, rb, y2);
+    if constexpr (Op::kCoefNeedsPrimal) bits = vec_coef_bits<Op, T>(V, col, r0, carry);
+    // backward: rs_bar of the last row gets the chunks below through suf.d (0 in the
+    // last chunk); cn is J_left of the row below.  Rows past the end carry ybar 0 and
+    // rs_bar 0 on.
+    T ra = suf.d[0], rb = W == 2 ? suf.d[W - 1] : T(0), cn = T(1);
+#pragma unroll 1
+    for (int q = kVecR - kVecU; q >= 0; q -= kVecU) {
+        T cf[kVecU], y1[kVecU], y2[kVecU];
+        vec_coefs<Op, T>(V, r0 + q, col, bits, q, cf);
+        vec_rows(V.ya, V, r0 + q, col, T(0), y1);
+        if constexpr (W == 2) vec_rows(V.yb, V, r0 + q, col, T(0), y2);
+#pragma unroll
+        for (int u = kVecU - 1; u >= 0; --u) {
+            ra = fma(cn, ra, y1[u]);
+            if constexpr (W == 2) rb = fma(cn, rb, y2[u]);
+            cn = cf[u];
+            s_r[((q + u) * W) * kVecOutBlock + threadIdx.x] = ra;
+            if constexpr (W == 2) s_r[((q + u) * W + 1) * kVecOutBlock + threadIdx.x] = rb;
         }
-        s_r[((r - r0) * W) * kVecOutBlock + threadIdx.x] = ra;
-        if constexpr (W == 2) s_r[((r - r0) * W + 1) * kVecOutBlock + threadIdx.x] = rb;
     }
     // forward: the primal prefix and the adjoints
-    T* abar = static_cast<T*>(V.abar);
-    T* bbar = static_cast<T*>(V.bbar);
+    T* abar = static_cast<T*>(V.abar) + r0 * V.d + col;
+    T* bbar = W == 2 ? static_cast<T*>(V.bbar) + r0 * V.d + col : nullptr;
     P prev = carry;
-    for (int64_t r = r0; r < r1; ++r) {
-        const int64_t i = r * V.d + col;
-        T av = T(0), bv = T(0);
+#pragma unroll 1
+    for (int q = 0; q < kVecR; q += kVecU) {
+        T a[kVecU], b[kVecU];
         if constexpr (kP) {
-            av = __ldg(static_cast<const T*>(V.a) + i);
-            if constexpr (W == 2) bv = __ldg(static_cast<const T*>(V.b) + i);
+            vec_rows(V.a, V, r0 + q, col, Op::pad_a(), a);
+            if constexpr (W == 2) vec_rows(V.b, V, r0 + q, col, T(0), b);
         }
-        const T q1 = s_r[((r - r0) * W) * kVecOutBlock + threadIdx.x];
-        const T q2 = W == 2 ? s_r[((r - r0) * W + 1) * kVecOutBlock + threadIdx.x] : T(0);
-        T o1 = T(0), o2 = T(0);
-        Op::vjp_right(prev, av, bv, q1, q2, o1, o2);
-        if constexpr (kP) prev = Op::pcomb(prev, Op::pelem(av, bv));
-        if (V.accumulate) {
-            abar[i] += o1;
-            if constexpr (W == 2) bbar[i] += o2;
-        } else {
-            abar[i] = o1;
-            if constexpr (W == 2) bbar[i] = o2;
+#pragma unroll
+        for (int u = 0; u < kVecU; ++u) {
+            if (r0 + q + u >= V.n) continue;
+            const T av = kP ? a[u] : T(0), bv = kP && W == 2 ? b[u] : T(0);
+            const T q1 = s_r[((q + u) * W) * kVecOutBlock + threadIdx.x];
+            const T q2 = W == 2 ? s_r[((q + u) * W + 1) * kVecOutBlock + threadIdx.x] : T(0);
+            T o1 = T(0), o2 = T(0);
+            Op::vjp_right(prev, av, bv, q1, q2, o1, o2);
+            if constexpr (kP) prev = Op::pcomb(prev, Op::pelem(av, bv));
+            T* oa = abar + (q + u) * V.d;
+            if (V.accumulate) {
+                *oa += o1;
+                if constexpr (W == 2) bbar[(q + u) * V.d] += o2;
+            } else {
+                *oa = o1;
+                if constexpr (W == 2) bbar[(q + u) * V.d] = o2;
+            }
         }
     }
 }
@@ -238,15 +295,16 @@ int run_vec(int64_t n, int64_t d, const void* a, const void* b, const void* ya, 
     V.aggL = w + sizeof(WsHeader) + round_up((size_t)V.C * d * sizeof(typename Op::P), 256);
     const dim3 g2((unsigned)((d + kVecBlock - 1) / kVecBlock), (unsigned)V.C);
     const dim3 g5((unsigned)((d + kVecOutBlock - 1) / kVecOutBlock), (unsigned)V.C);
-    const unsigned gw = (unsigned)((d + 7) / 8);  // 8 warps (columns) per block
-    if constexpr (kVecPrimal<Op>) {
-        vec_primal_agg_kernel<Op, T><<<g2, kVecBlock, 0, s>>>(V);
-        vec_scan_P_kernel<Op, T><<<gw, 256, 0, s>>>(V);
+    const unsigned gw = (unsigned)((d + 31) / 32);  // 32 columns per block
+    const size_t sh = std::max(sizeof(typename Op::P), sizeof(L)) * 32 * kVecG;
+    constexpr bool kTwo = kVecPrimal<Op> && !Op::kCoefNeedsPrimal;  // both aggregates from one launch
+    if constexpr (Op::kCoefNeedsPrimal) {
+        vec_agg_kernel<Op, T, true, false><<<g2, kVecBlock, 0, s>>>(V);
+        vec_scan_kernel<Op, T><<<dim3(gw, 1), 32 * kVecG, sh, s>>>(V, 0);
     }
-    vec_adjoint_agg_kernel<Op, T><<<g2, kVecBlock, 0, s>>>(V);
-    vec_scan_L_kernel<Op, T><<<gw, 256, 0, s>>>(V);
+    vec_agg_kernel<Op, T, kTwo, true><<<g2, kVecBlock, 0, s>>>(V);
+    vec_scan_kernel<Op, T><<<dim3(gw, kTwo ? 2 : 1), 32 * kVecG, sh, s>>>(V, kTwo ? 0 : 1);
     vec_output_kernel<Op, T><<<g5, kVecOutBlock, 0, s>>>(V);
-    (void)sizeof(L);
     return cudaGetLastError() == cudaSuccess ? ADPAR_OK : ADPAR_ERR_CUDA;
 }
 
