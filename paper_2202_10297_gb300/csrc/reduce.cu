@@ -200,6 +200,23 @@ __global__ void __launch_bounds__(kRedBlock) reduce_arg_kernel(ReduceArgs A) {
 }
 
 // ------------------------------------------------------------------ MUL
+// y and the product record of a finished product
+template <class T>
+__device__ __forceinline__ void prod_results(const ReduceArgs& A, const ProdState& tot) {
+    if (A.y_out) *static_cast<T*>(A.y_out) = tot.nz > 0 ? T(0) : (T)ldexp_clamped(tot.m, tot.e);
+    if (A.aux_out) {
+        adpar_prod_aux x;
+        x.nzero = tot.nz;
+        x.first_zero = tot.nz > 0 ? tot.first : -1;
+        x.exp2 = tot.e;
+        x.mant = tot.m;
+        x.log_abs_nz = log(fabs(tot.m)) + (double)tot.e * 0.69314718055994530942;
+        x.sign = tot.m > 0 ? 1 : -1;
+        x.reserved = 0;
+        *A.aux_out = x;
+    }
+}
+
 // The recompute multiplies mantissas in fixed point on the integer pipes
 // (no FP64 instruction per element for either dtype).
 template <class T>
@@ -243,19 +260,7 @@ __global__ void __launch_bounds__(kRedBlock, 4) reduce_prod_kernel(ReduceArgs A)
     if (threadIdx.x == 0) {
         const ProdState tot = totq.to_state();
         *static_cast<ProdState*>(A.final_state) = tot;
-        if (A.y_out)
-            *static_cast<T*>(A.y_out) = tot.nz > 0 ? T(0) : (T)ldexp_clamped(tot.m, tot.e);
-        if (A.aux_out) {
-            adpar_prod_aux x;
-            x.nzero = tot.nz;
-            x.first_zero = tot.nz > 0 ? tot.first : -1;
-            x.exp2 = tot.e;
-            x.mant = tot.m;
-            x.log_abs_nz = log(fabs(tot.m)) + (double)tot.e * 0.69314718055994530942;
-            x.sign = tot.m > 0 ? 1 : -1;
-            x.reserved = 0;
-            *A.aux_out = x;
-        }
+        prod_results<T>(A, tot);
         A.hdr->done[0] = 0u;
     }
 }
@@ -276,11 +281,10 @@ __device__ __forceinline__ void prod_adjoint_body(const ReduceArgs& A, const Pro
     double ym = 0.0;
     int64_t ye = 0;
     if (yb != 0.0) split_pow2(yb, ym, ye);
-    const double lg_p = log(fabs(st.m)) + (double)st.e * 0.69314718055994530942;
-    const double lg_y = yb != 0.0 ? log(fabs(yb)) : -CUDART_INF;
-    const int sgn_py = (st.m > 0 ? 1 : -1) * (yb > 0 ? 1 : (yb < 0 ? -1 : 0));
-
     if (A.logdomain) {
+        const double lg_p = log(fabs(st.m)) + (double)st.e * 0.69314718055994530942;
+        const double lg_y = yb != 0.0 ? log(fabs(yb)) : -CUDART_INF;
+        const int sgn_py = (st.m > 0 ? 1 : -1) * (yb > 0 ? 1 : (yb < 0 ? -1 : 0));
         for (int64_t i = t0; i < A.n; i += stride) {
             double lg = -CUDART_INF;
             int sg = 0;
@@ -364,6 +368,82 @@ __global__ void __launch_bounds__(kRedBlock, 4) prod_adjoint_kernel(ReduceArgs A
     prod_adjoint_body<T>(A, st, blockIdx.x * (int64_t)blockDim.x + threadIdx.x, (int64_t)gridDim.x * blockDim.x);
 }
 
+// ------------------------------------------------------ one-cluster form
+// Short arrays: the whole call in one launch of one cluster of 8 blocks.  Each
+// block reduces its share, the blocks read each other's states through
+// distributed shared memory (a hardware barrier of the cluster instead of a
+// global counter that an earlier launch must clear), and every block maps its
+// share with the same total.  65536 FP64 values: 11 us on the device against 17 in
+// three launches (and their gaps), 29.5 against 35.6 us per call from Python; at 2 MB
+// 28 against 32, at 4 MB 45 against 32.
+constexpr int kClusterBlocks = 8;
+constexpr int kClusterThreads = 1024;
+constexpr int64_t kClusterBytes = int64_t(2) << 20;
+
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+// block `rank`'s copy of the shared variable at p
+template <class S>
+__device__ __forceinline__ S ld_cluster(const S* p, unsigned rank) {
+    static_assert(sizeof(S) % 8 == 0, "8-byte granules");
+    constexpr int N = sizeof(S) / 8;
+    union {
+        S s;
+        unsigned long long w[N];
+    } u;
+    unsigned a;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"((unsigned)__cvta_generic_to_shared(p)), "r"(rank));
+#pragma unroll
+    for (int i = 0; i < N; ++i)
+        asm volatile("ld.shared::cluster.u64 %0, [%1];" : "=l"(u.w[i]) : "r"(a + 8u * i));
+    return u.s;
+}
+
+template <class T>
+__global__ void __cluster_dims__(kClusterBlocks, 1, 1) __launch_bounds__(kClusterThreads, 1)
+    reduce_prod_cluster_kernel(ReduceArgs A) {
+    using S = ProdStateQ;
+    __shared__ S s_warp[kClusterThreads / 32];
+    __shared__ S s_block;
+    __shared__ ProdState s_total;
+    const T* a = static_cast<const T*>(A.a);
+    constexpr int V = Vec16<T>::N, U = 4;
+    const int64_t nvec = A.n / V, stride = kClusterBlocks * kClusterThreads;
+    const int64_t t0 = blockIdx.x * (int64_t)kClusterThreads + threadIdx.x;
+    if (t0 < 64) reinterpret_cast<uint32_t*>(A.hdr)[t0] = 0u;  // the status word starts at ok
+    ProdAcc st = ProdAcc::id();
+    for (int64_t v0 = t0; v0 < nvec; v0 += U * stride) {
+        Vec16<T> x[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (v0 + u * stride < nvec) x[u] = ld_vec(a + (v0 + u * stride) * V);
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (v0 + u * stride >= nvec) break;
+#pragma unroll
+            for (int j = 0; j < V; ++j) st.push(x[u].v[j], (v0 + u * stride) * V + j);
+        }
+    }
+    if (t0 < A.n - nvec * V) st.push(a[nvec * V + t0], nvec * V + t0);
+    auto comb = [](const S& x, const S& y) { return S::comb(x, y); };
+    const S bs = block_reduce(st.state(), comb, s_warp);
+    if (threadIdx.x == 0) s_block = bs;
+    cluster_sync();
+    if (threadIdx.x < 32) {
+        S q = (int)threadIdx.x < kClusterBlocks ? ld_cluster(&s_block, threadIdx.x) : S::id();
+#pragma unroll
+        for (int off = kClusterBlocks / 2; off > 0; off >>= 1) q = S::comb(q, shfl_down_s(q, off));
+        if (threadIdx.x == 0) {
+            s_total = q.to_state();
+            if (blockIdx.x == 0) prod_results<T>(A, s_total);
+        }
+    }
+    __syncthreads();
+    if (!A.primal_only) prod_adjoint_body<T>(A, s_total, t0, stride);
+    cluster_sync();  // no block leaves while another may read its state
+}
+
 // ------------------------------------------------------------ host side
 size_t state_bytes(int op, int dtype) {
     const size_t t = dtype == ADPAR_F64 ? 8 : 4;
@@ -388,6 +468,10 @@ int grid_for(int64_t n, int dtype) {
 template <class T>
 int run_reduce(ReduceArgs A, int op, cudaStream_t s) {
     const int grid = grid_for(A.n, sizeof(T) == 8 ? ADPAR_F64 : ADPAR_F32);
+    // the "last block" counter must start at zero in a workspace of unknown
+    // contents
+    const bool cluster = op == ADPAR_OP_MUL && A.n * (int64_t)sizeof(T) <= kClusterBytes;
+    if (!cluster) header_init_kernel<<<1, 64, 0, s>>>(A.hdr);
     switch (op) {
     case ADPAR_OP_ADD:
         reduce_add_kernel<T><<<grid, kRedBlock, 0, s>>>(A);
@@ -399,6 +483,10 @@ int run_reduce(ReduceArgs A, int op, cudaStream_t s) {
         reduce_arg_kernel<T, true><<<grid, kRedBlock, 0, s>>>(A);
         break;
     case ADPAR_OP_MUL: {
+        if (cluster) {
+            reduce_prod_cluster_kernel<T><<<kClusterBlocks, kClusterThreads, 0, s>>>(A);
+            break;
+        }
         // one 16-byte vector per thread, up to a whole wave of resident blocks
         const int64_t per = (int64_t)kRedBlock * (16 / sizeof(T));
         const int gp = (int)std::max<int64_t>(1, std::min<int64_t>((A.n + per - 1) / per, kProdGrid));
@@ -459,9 +547,6 @@ extern "C" int adpar_vjp_reduce(adpar_opdesc d, int64_t n, const void* a, const 
     A.partials = w + sizeof(WsHeader);
     A.final_state = w + sizeof(WsHeader) + round_up(kRedMaxBlocks * state_bytes(d.op, d.dtype), 256);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    // the "last block" counter must start at zero in a workspace of unknown
-    // contents
-    header_init_kernel<<<1, 64, 0, s>>>(A.hdr);
     if (d.dtype == ADPAR_F32) return run_reduce<float>(A, d.op, s);
     return run_reduce<double>(A, d.op, s);
 }
@@ -490,7 +575,6 @@ extern "C" int adpar_reduce(adpar_opdesc d, int64_t n, const void* a, void* y_ou
     A.partials = w + sizeof(WsHeader);
     A.final_state = w + sizeof(WsHeader) + round_up(kRedMaxBlocks * state_bytes(d.op, d.dtype), 256);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    header_init_kernel<<<1, 64, 0, s>>>(A.hdr);
     if (d.dtype == ADPAR_F32) return run_reduce<float>(A, d.op, s);
     return run_reduce<double>(A, d.op, s);
 }

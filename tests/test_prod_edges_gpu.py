@@ -75,3 +75,29 @@ def test_sizes(dt, rel, n, accumulate):
         assert np.all(np.abs(got - (0.5 + ref)) <= (np.abs(ref) + 1.0) * 2 * rel)
     else:
         assert np.all(np.abs(got - ref) <= np.abs(ref) * rel * (1 + n * 2.0 ** -14 * (dt == np.float64)))
+
+
+# one cluster of 8 x 1024 threads up to 2 MB, three launches beyond
+@pytest.mark.parametrize("dt", [np.float64, np.float32])
+@pytest.mark.parametrize("over", [-1, 0, 1])
+@pytest.mark.parametrize("zeros", [0, 1, 2])
+def test_one_cluster_boundary(dt, over, zeros):
+    from paper_2202_10297_gb300 import adpar as A
+    n = (2 << 20) // np.dtype(dt).itemsize + over
+    g = np.random.default_rng(n + zeros)
+    a = np.exp(g.uniform(-2.0 ** -10, 2.0 ** -10, n)).astype(dt)
+    pos = np.sort(g.choice(n, zeros, replace=False))
+    nz = np.delete(a, pos)
+    a[pos] = 0
+    p = _product(nz)[0]
+    out = A.adpar_vjp_reduce("mul", torch.from_numpy(a).cuda(), 1.25, want_y=True, want_aux=True)
+    assert out["aux"].nzero == zeros and out["aux"].first_zero == (pos[0] if zeros else -1)
+    rel = 2.0 ** -47 if dt == np.float64 else 2.0 ** -22
+    got = out["abar"].cpu().numpy().astype(np.float64)
+    ref = 1.25 * p / a.astype(np.float64) if zeros == 0 else np.zeros(n)
+    if zeros == 1:
+        ref[pos[0]] = 1.25 * p
+    assert np.all(np.abs(got - ref) <= rel * np.abs(ref))
+    assert A.adpar_workspace_status(out["work"]) == A.OK
+    lg = A.adpar_vjp_reduce("mul", torch.from_numpy(a).cuda(), 1.25, logdomain=True)["abar"].cpu().numpy()
+    assert np.array_equal(np.isfinite(lg), ref != 0)
