@@ -1238,6 +1238,55 @@ int run_scan_forward(int64_t n, const void* a, const void* b, void* ys_a, void* 
     return cudaGetLastError() == cudaSuccess ? ADPAR_OK : ADPAR_ERR_CUDA;
 }
 
+// the linear recurrence on per-thread runs (scan_runs.cuh); its tiles are the
+// scan engine's, so the engine's primal slots serve it
+template <class T>
+int run_linrec_runs_scan(int64_t n, const void* a, const void* b, void* ys_a, void* ys_b, void* work,
+                         size_t work_bytes, cudaStream_t stream) {
+    using Cf = RunCfg<T>;
+    using Op = OpLinrec<T>;
+    static_assert(Cf::TILE == ScanCfg<Op, T>::TILE, "runs tiles are the engine's tiles");
+    static_assert(lb_words<RunP<T>>() == lb_words<typename Op::P>(), "primal slots");
+    const ScanLayout L = scan_layout<Op, T>(n);
+    if (work == nullptr || work_bytes < L.total_min || (reinterpret_cast<uintptr_t>(work) & 255u))
+        return ADPAR_ERR_WORKSPACE;
+    if (n == 0) return ADPAR_OK;
+    char* w = static_cast<char*>(work);
+    RunScanArgs<T> R{};
+    R.n = n;
+    R.tiles = (n + Cf::TILE - 1) / Cf::TILE;
+    R.a = static_cast<const T*>(a);
+    R.b = static_cast<const T*>(b);
+    R.ys_a = static_cast<T*>(ys_a);
+    R.ys_b = static_cast<T*>(ys_b);
+    R.hdr = reinterpret_cast<WsHeader*>(w);
+    R.lb_agg = reinterpret_cast<unsigned long long*>(w + L.off_pA);
+    R.lb_incl = reinterpret_cast<unsigned long long*>(w + L.off_pI);
+    CUtensorMap tm[4];
+    memset(tm, 0, sizeof(tm));
+    if (n >= Cf::TILE) {
+        const T* ptr[4] = {R.a, R.b, R.ys_a, R.ys_b};
+        for (int i = 0; i < 4; ++i)
+            if (!make_run_map<T>(&tm[i], ptr[i], n)) return ADPAR_ERR_CUDA;
+    }
+    static bool configured[64] = {};
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return ADPAR_ERR_CUDA;
+    if (!configured[dev]) {
+        if (cudaFuncSetAttribute(linrec_runs_scan_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 2 * Cf::ARR) != cudaSuccess)
+            return ADPAR_ERR_CUDA;
+        configured[dev] = true;
+    }
+    ScanArgs A{};
+    A.hdr = R.hdr;
+    A.tiles = R.tiles;
+    set_slots(A, w, L);
+    launch_init(A, w, L, stream);
+    linrec_runs_scan_kernel<T><<<(unsigned)R.tiles, Cf::NT, 2 * Cf::ARR, stream>>>(tm[0], tm[1], tm[2], tm[3], R);
+    return cudaGetLastError() == cudaSuccess ? ADPAR_OK : ADPAR_ERR_CUDA;
+}
+
 template <class T>
 int dispatch_scan_forward(int op, int64_t n, const void* a, const void* b, void* ys_a, void* ys_b,
                           void* work, size_t work_bytes, cudaStream_t s) {
@@ -1246,7 +1295,7 @@ int dispatch_scan_forward(int op, int64_t n, const void* a, const void* b, void*
     case ADPAR_OP_MUL: return run_scan_forward<OpMul<T>, T>(n, a, b, ys_a, ys_b, work, work_bytes, s);
     case ADPAR_OP_MIN: return run_scan_forward<OpMin<T>, T>(n, a, b, ys_a, ys_b, work, work_bytes, s);
     case ADPAR_OP_MAX: return run_scan_forward<OpMax<T>, T>(n, a, b, ys_a, ys_b, work, work_bytes, s);
-    case ADPAR_OP_LINREC: return run_scan_forward<OpLinrec<T>, T>(n, a, b, ys_a, ys_b, work, work_bytes, s);
+    case ADPAR_OP_LINREC: return run_linrec_runs_scan<T>(n, a, b, ys_a, ys_b, work, work_bytes, s);
     }
     return ADPAR_ERR_INVALID;
 }

@@ -567,6 +567,124 @@ __global__ void __launch_bounds__(RunCfg<T>::NT) linrec_runs_jvp_kernel(
 
 }  // namespace adpar
 
+// ------------------------------------------------- forward operator
+// The inclusive scan itself, one single pass on per-thread runs: a tile folds
+// each run (2 operations per element), scans the runs, looks back over the
+// earlier tiles, re-folds every run from its exclusive carry over the inputs
+// (2 more) and leaves by TMA.  FP64 is bound by the FP64 pipe (about 5
+// instructions per pair), FP32 by HBM.  FIGURES
+namespace adpar {
+
+template <class T>
+struct RunScanArgs {
+    int64_t n;
+    int64_t tiles;
+    const T* a;
+    const T* b;
+    T* ys_a;
+    T* ys_b;
+    WsHeader* hdr;
+    unsigned long long* lb_agg;
+    unsigned long long* lb_incl;
+};
+
+template <class T>
+__global__ void __launch_bounds__(RunCfg<T>::NT, 6) linrec_runs_scan_kernel(
+    const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
+    const __grid_constant__ CUtensorMap tmYA, const __grid_constant__ CUtensorMap tmYB, RunScanArgs<T> R) {
+    using Cf = RunCfg<T>;
+    using P = RunP<T>;
+    constexpr int EPC = Cf::EPC;
+    extern __shared__ __align__(1024) unsigned char s_dyn[];
+    unsigned char* sA = s_dyn;            // a, then ys_a
+    unsigned char* sB = s_dyn + Cf::ARR;  // b, then ys_b
+    __shared__ __align__(8) uint64_t s_bar;
+    __shared__ uint32_t s_tile;
+    __shared__ P s_tot[Cf::NW];
+    if (threadIdx.x == 0) s_tile = atomicAdd(&R.hdr->ticket[0], 1u);
+    __syncthreads();
+    const int64_t tile = s_tile;
+    const bool whole = (tile + 1) * Cf::TILE <= R.n;
+    const int t = threadIdx.x;
+    if (t == 0 && (tile + kRunAheadC + 1) * Cf::TILE <= R.n) {
+        const int64_t e = (tile + kRunAheadC) * Cf::TILE;
+        tc::prefetch_l2(R.a + e, Cf::ARR);
+        tc::prefetch_l2(R.b + e, Cf::ARR);
+    }
+    {
+        unsigned char* const dst[2] = {sA, sB};
+        const CUtensorMap* const tm[2] = {&tmA, &tmB};
+        const T* const src[2] = {R.a, R.b};
+        const T pad[2] = {T(1), T(0)};  // the identity element
+        run_tile_load<T, 2>(dst, tm, src, pad, whole, tile, R.n, &s_bar, R.hdr);
+    }
+    const P ident{T(1), T(0)};
+    auto push = [](P& s, T x, T y) {
+        s.B = run_fma(x, s.B, y);
+        s.A = x * s.A;
+    };
+    P run = ident;
+#pragma unroll
+    for (int p = 0; p < kRunChunks; ++p) {
+        const int off = run_chunk_off(t, p);
+        const RunVec<T> x = run_ld<T>(sA, off), y = run_ld<T>(sB, off);
+#pragma unroll
+        for (int j = 0; j < EPC; ++j) push(run, x.v[j], y.v[j]);
+    }
+    auto comb = [](const P& l, const P& r) { return RunPOp<T>::pcomb(l, r); };
+    const P agg[1] = {run};
+    P wex[1];
+    const P total = block_scan_part1<P, false, 1, Cf::NW>(agg, wex, s_tot, ident, comb);
+    if ((threadIdx.x >> 5) == 0) {
+        LookbackState<P> st{R.lb_agg, R.lb_incl};
+        const P pre = lookback(tile, st, total, ident, comb, R.hdr);
+        block_fold_prefix<P, 1, Cf::NW>(s_tot, pre, comb);
+    }
+    __syncthreads();
+    P s = block_scan_excl_folded<P, false, 1, Cf::NW>(0, wex, s_tot, comb);
+#pragma unroll
+    for (int p = 0; p < kRunChunks; ++p) {
+        const int off = run_chunk_off(t, p);
+        const RunVec<T> x = run_ld<T>(sA, off), y = run_ld<T>(sB, off);
+        RunVec<T> oA, oB;
+#pragma unroll
+        for (int j = 0; j < EPC; ++j) {
+            push(s, x.v[j], y.v[j]);
+            oA.v[j] = s.A;
+            oB.v[j] = s.B;
+        }
+        run_st<T>(sA, off, oA);
+        run_st<T>(sB, off, oB);
+    }
+    if (whole) {
+        tc::fence_proxy_async();
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            tma_store_3d(&tmYA, (int)(tile * Cf::NT), sA);
+            tma_store_3d(&tmYB, (int)(tile * Cf::NT), sB);
+            bulk_commit_and_wait_read();
+        }
+        __syncthreads();
+    } else {
+        const int64_t e0 = tile * Cf::TILE + (int64_t)t * Cf::V;
+#pragma unroll 2
+        for (int p = 0; p < kRunChunks; ++p) {
+            const int off = run_chunk_off(t, p);
+            const RunVec<T> oA = run_ld<T>(sA, off), oB = run_ld<T>(sB, off);
+#pragma unroll
+            for (int j = 0; j < EPC; ++j) {
+                const int64_t e = e0 + EPC * p + j;
+                if (e < R.n) {
+                    R.ys_a[e] = oA.v[j];
+                    R.ys_b[e] = oB.v[j];
+                }
+            }
+        }
+    }
+}
+
+}  // namespace adpar
+
 // --------------------------------------- reduce VJP, general rule (LINREC)
 // The VJP of y = reduce (.) as for the linear recurrence by the general rule
 // of Sec. 5.1: with l_i the composite of the elements before i and r_i of
