@@ -94,23 +94,24 @@ __global__ void __launch_bounds__(kScanBlock) scan_tile_agg_kernel(ScanArgs A, t
     if (threadIdx.x == 0) agg[tile] = total;
 }
 
-// carry[i] = agg[0] (.) ... (.) agg[i-1], in order, over segments of
-// kCarrySeg tiles: carry_local_kernel scans each segment (one block per
-// segment) and writes its total, carry_apply_kernel puts the fold of the
-// earlier segments' totals in front.  (One block over every tile left the
-// FP64 combines to one SM: 116 us for 32768 FP64 tiles.)  segtot holds one
-// state per segment.
-constexpr int kCarryBlock = 1024;
+// carry[i] = agg[0] (.) ... (.) agg[i-1], in order, over segments of B * kCarryPer
+// tiles: carry_local_kernel scans each segment (one block of B threads) and
+// writes its total, carry_apply_kernel puts the fold of the earlier segments'
+// totals in front.  The combines of a segment queue on one SM's FP64 pipe, so
+// many tiles take short segments: one block over every tile took 116 us for
+// 32768 FP64 tiles; for 4883, segments of 4096 take 13 + 7 us, of 512 4 + 6.
+// Few tiles take one segment and no second launch (FP32 to 4096 tiles, 8 us;
+// FP64 to 1024).  segtot holds one state per segment.
 constexpr int kCarryPer = 4;
-constexpr int kCarrySeg = kCarryBlock * kCarryPer;
+constexpr int kCarryShort = 128;  // B of the segmented form
 
-template <class Op>
-__global__ void __launch_bounds__(kCarryBlock) carry_local_kernel(const typename Op::P* agg, typename Op::P* carry,
+template <class Op, int B>
+__global__ void __launch_bounds__(B) carry_local_kernel(const typename Op::P* agg, typename Op::P* carry,
                                                                   typename Op::P* segtot, int64_t tiles) {
     using P = typename Op::P;
-    __shared__ P s_w[kCarryBlock / 32];
+    __shared__ P s_w[B / 32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int64_t base = (int64_t)blockIdx.x * kCarrySeg + (int64_t)threadIdx.x * kCarryPer;
+    const int64_t base = (int64_t)blockIdx.x * (B * kCarryPer) + (int64_t)threadIdx.x * kCarryPer;
     P v[kCarryPer];
     P run = Op::pid();
 #pragma unroll
@@ -127,13 +128,14 @@ __global__ void __launch_bounds__(kCarryBlock) carry_local_kernel(const typename
     if (lane == 31) s_w[warp] = inc;
     __syncthreads();
     if (warp == 0) {
-        P w = s_w[lane];
+        constexpr int NW = B / 32;
+        P w = lane < NW ? s_w[lane] : Op::pid();
 #pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
+        for (int off = 1; off < NW; off <<= 1) {
             const P o = shfl_up_s(w, off);
             if (lane >= off) w = Op::pcomb(o, w);
         }
-        s_w[lane] = w;
+        if (lane < NW) s_w[lane] = w;
     }
     __syncthreads();
     P ex = shfl_up_s(inc, 1);
@@ -144,13 +146,14 @@ __global__ void __launch_bounds__(kCarryBlock) carry_local_kernel(const typename
         if (base + j < tiles) carry[base + j] = ex;
         ex = Op::pcomb(ex, v[j]);
     }
-    if (threadIdx.x == 0) segtot[blockIdx.x] = s_w[kCarryBlock / 32 - 1];
+    if (threadIdx.x == 0) segtot[blockIdx.x] = s_w[B / 32 - 1];
 }
 
 template <class Op>
-__global__ void __launch_bounds__(256) carry_apply_kernel(typename Op::P* carry, const typename Op::P* segtot,
+__global__ void __launch_bounds__(kCarryShort) carry_apply_kernel(typename Op::P* carry, const typename Op::P* segtot,
                                                           int64_t tiles) {
     using P = typename Op::P;
+    constexpr int64_t kSeg = kCarryShort * kCarryPer;
     if (blockIdx.x == 0) return;
     __shared__ P s_pre;
     if (threadIdx.x < 32) {
@@ -169,19 +172,29 @@ __global__ void __launch_bounds__(256) carry_apply_kernel(typename Op::P* carry,
     }
     __syncthreads();
     const P pre = s_pre;
-    const int64_t lo = (int64_t)blockIdx.x * kCarrySeg;
-    const int64_t hi = lo + kCarrySeg < tiles ? lo + kCarrySeg : tiles;
+    const int64_t lo = (int64_t)blockIdx.x * kSeg;
+    const int64_t hi = lo + kSeg < tiles ? lo + kSeg : tiles;
     for (int64_t i = lo + threadIdx.x; i < hi; i += blockDim.x) carry[i] = Op::pcomb(pre, carry[i]);
 }
 
 // the tile carries from the tile aggregates; segtot: room for one state per
-// kCarrySeg tiles
-template <class Op>
+// segment
+template <class Op, class T>
 void launch_carry_scan(const typename Op::P* agg, typename Op::P* carry, typename Op::P* segtot, int64_t tiles,
                        cudaStream_t stream) {
-    const unsigned nseg = (unsigned)((tiles + kCarrySeg - 1) / kCarrySeg);
-    carry_local_kernel<Op><<<nseg, kCarryBlock, 0, stream>>>(agg, carry, segtot, tiles);
-    if (nseg > 1) carry_apply_kernel<Op><<<nseg, 256, 0, stream>>>(carry, segtot, tiles);
+    constexpr bool kF64 = sizeof(T) == 8;
+    const int64_t seg = kCarryShort * kCarryPer;
+    if (tiles <= seg) {
+        carry_local_kernel<Op, kCarryShort><<<1, kCarryShort, 0, stream>>>(agg, carry, segtot, tiles);
+    } else if (tiles <= 1024) {
+        carry_local_kernel<Op, 256><<<1, 256, 0, stream>>>(agg, carry, segtot, tiles);
+    } else if (!kF64 && tiles <= 4096) {
+        carry_local_kernel<Op, 1024><<<1, 1024, 0, stream>>>(agg, carry, segtot, tiles);
+    } else {
+        const unsigned nseg = (unsigned)((tiles + seg - 1) / seg);
+        carry_local_kernel<Op, kCarryShort><<<nseg, kCarryShort, 0, stream>>>(agg, carry, segtot, tiles);
+        carry_apply_kernel<Op><<<nseg, kCarryShort, 0, stream>>>(carry, segtot, tiles);
+    }
 }
 
 // MIN/MAX scans: the return sweep fused into the forward pass.  For these
@@ -962,7 +975,7 @@ int runs_carry_pass(int64_t n, const void* a, const void* b, const void* ya, con
     linrec_runs_carry_kernel<T><<<(unsigned)L.tiles, Cf::NT, 2 * Cf::ARR, stream>>>(tm[0], tm[1], R);
     // the segment totals take the second half of the tile aggregates' slots
     static_assert(lb_words<RunP<T>>() * 8 >= 2 * sizeof(RunP<T>), "room after the aggregates");
-    launch_carry_scan<RunPOp<T>>(R.tagg, R.tcar, R.tagg + L.tiles, L.tiles, stream);
+    launch_carry_scan<RunPOp<T>, T>(R.tagg, R.tcar, R.tagg + L.tiles, L.tiles, stream);
     return ADPAR_OK;
 }
 
@@ -1177,7 +1190,7 @@ int run_scan(int64_t n, const void* a, const void* b, const void* ya, const void
             static_assert(lb_words<P>() * 8 >= 2 * sizeof(P), "an aggregate and a total fit a slot");
             P* agg = reinterpret_cast<P*>(A.lbP_agg);
             scan_tile_agg_kernel<Op, T><<<(unsigned)A.tiles, kScanBlock, 0, stream>>>(A, agg);
-            launch_carry_scan<Op>(agg, static_cast<P*>(A.carry), agg + A.tiles, A.tiles, stream);
+            launch_carry_scan<Op, T>(agg, static_cast<P*>(A.carry), agg + A.tiles, A.tiles, stream);
         }
         if (ys_a) scan_adjoint_kernel<Op, T, true><<<(unsigned)A.tiles, kScanBlock, 0, stream>>>(A);
         else scan_adjoint_kernel<Op, T, false><<<(unsigned)A.tiles, kScanBlock, 0, stream>>>(A);
