@@ -3,15 +3,17 @@
 // (Sec. 5.2), in ONE persistent launch that a CUDA graph can capture.
 //
 // Work items.  Segment s of length L has R = ceil(L / RT) reduce tiles and
-// S = ceil(L / ST) scan tiles, and contributes, in this order,
-//   R product-reduce tiles, S primal-scan tiles (left to right),
-//   S adjoint-scan tiles (right to left), R product-map tiles.
-// Items are numbered segment after segment and handed out by one global
-// atomic ticket.  An item only ever waits on items with smaller numbers of
-// its own segment (the look-back predecessors, the primal carries, the
-// finished product), which were handed out earlier to blocks that are
-// running, so the schedule cannot deadlock, and every wait is bounded.
-// Small segments are one tile of each kind; no look-back happens there.
+// S = ceil(L / ST) scan tiles, and contributes two parts:
+//   A  R product-reduce tiles, S primal-scan tiles (left to right),
+//   B  S adjoint-scan tiles (right to left), R product-map tiles.
+// Items are numbered A(0), A(1) B(0), A(2) B(1), .. and handed out by one global
+// atomic ticket, so that a segment's return sweep comes up when its forward
+// sweep, one segment earlier, is done rather than just begun.  An item only
+// ever waits on items with smaller numbers of its own segment (the look-back
+// predecessors, the primal carries, the finished product), which were handed
+// out earlier to blocks that are running, so the schedule cannot deadlock, and
+// every wait is bounded.  Small segments are one tile of each kind; no
+// look-back happens there.
 //
 // The scan tiles run the linear recurrence on per-thread runs
 // (batch_runs.cuh: a forward tile stores its runs' carries, a reverse tile
@@ -43,7 +45,7 @@ struct BatchPlanHeader {
 };
 
 struct SegMeta {
-    int64_t item_base;  // first item number of the segment
+    int64_t item_base;  // first item number of the segment's part A
     int64_t state_off;  // byte offset of its state in the workspace
     int32_t red_tiles;
     int32_t scan_tiles;
@@ -87,18 +89,19 @@ __host__ __device__ inline StateLayout state_layout(int dtype, int red, int scan
 }
 
 template <class S>
-__device__ __forceinline__ S block_reduce_256(S v, S (*comb)(const S&, const S&), S* s_warp) {
+__device__ __forceinline__ S block_reduce_bnt(S v, S (*comb)(const S&, const S&), S* s_warp) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) v = comb(v, shfl_down_s(v, off));
     if (lane == 0) s_warp[warp] = v;
     __syncthreads();
     if (warp == 0) {
-        v = s_warp[lane < 8 ? lane : 0];
+        constexpr int NW = kBNT / 32;
+        v = s_warp[lane < NW ? lane : 0];
 #pragma unroll
-        for (int off = 4; off > 0; off >>= 1) {
+        for (int off = NW / 2; off > 0; off >>= 1) {
             S o = shfl_down_s(v, off);
-            if (lane + off < 8) v = comb(v, o);
+            if (lane + off < NW) v = comb(v, o);
         }
     }
     return v;  // valid in thread 0
@@ -110,23 +113,32 @@ __device__ ProdStateQ prod_comb(const ProdStateQ& x, const ProdStateQ& y) { retu
 template <class T>
 __device__ void prod_reduce_tile(const adpar_batch_segment& sg, char* st, const StateLayout& L, int red, int r,
                                  int RT, WsHeader* hdr) {
-    __shared__ ProdStateQ s_warp[8];
+    __shared__ ProdStateQ s_warp[kBNT / 32];
     __shared__ int s_last;
     const T* x = static_cast<const T*>(sg.x);
     const int64_t lo = (int64_t)r * RT, hi = std::min<int64_t>(sg.len, lo + RT);
     range_prefetch_l2(x, lo, hi);
     ProdAcc ps = ProdAcc::id();  // fixed-point products: no FP64 per element
     constexpr int V = Vec16<T>::N;
-    for (int64_t i = lo + threadIdx.x * V; i < hi; i += 256 * V) {
-        if (i + V <= hi) {
-            Vec16<T> v = ld_vec(x + i);
+    constexpr int U = 4;  // vectors in flight per thread
+    const int64_t whole = lo + (hi - lo) / V * V;
+    int64_t i = lo + threadIdx.x * V;
+    for (; i + (U - 1) * kBNT * V < whole; i += U * kBNT * V) {
+        Vec16<T> v[U];
 #pragma unroll
-            for (int j = 0; j < V; ++j) ps.push(v.v[j], i + j);
-        } else {
-            for (int64_t j = i; j < hi; ++j) ps.push(x[j], j);
-        }
+        for (int u = 0; u < U; ++u) v[u] = ld_vec(x + i + u * kBNT * V);
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+#pragma unroll
+            for (int j = 0; j < V; ++j) ps.push(v[u].v[j], i + u * kBNT * V + j);
     }
-    ProdStateQ bs = block_reduce_256<ProdStateQ>(ps.state(), prod_comb, s_warp);
+    for (; i < whole; i += kBNT * V) {
+        const Vec16<T> v = ld_vec(x + i);
+#pragma unroll
+        for (int j = 0; j < V; ++j) ps.push(v.v[j], i + j);
+    }
+    if (whole + threadIdx.x < hi) ps.push(x[whole + threadIdx.x], whole + threadIdx.x);
+    ProdStateQ bs = block_reduce_bnt<ProdStateQ>(ps.state(), prod_comb, s_warp);
     ProdStateQ* partials = reinterpret_cast<ProdStateQ*>(st + L.partials);
     unsigned int* counter = reinterpret_cast<unsigned int*>(st + L.counter);
     if (threadIdx.x == 0) {
@@ -138,9 +150,9 @@ __device__ void prod_reduce_tile(const adpar_batch_segment& sg, char* st, const 
     if (!s_last) return;
     __threadfence();
     ProdStateQ totq = ProdStateQ::id();
-    for (int q = threadIdx.x; q < red; q += 256) totq = ProdStateQ::comb(totq, ld_cg(partials + q));
+    for (int q = threadIdx.x; q < red; q += kBNT) totq = ProdStateQ::comb(totq, ld_cg(partials + q));
     __syncthreads();
-    totq = block_reduce_256<ProdStateQ>(totq, prod_comb, s_warp);
+    totq = block_reduce_bnt<ProdStateQ>(totq, prod_comb, s_warp);
     if (threadIdx.x == 0) {
         const ProdState tot = totq.to_state();
         *reinterpret_cast<ProdState*>(st + L.final_state) = tot;
@@ -193,15 +205,15 @@ __device__ void prod_map_tile(const adpar_batch_segment& sg, char* st, const Sta
         constexpr int V = Vec16<T>::N;
         const int64_t whole = lo + (hi - lo) / V * V;
         int64_t i = lo + threadIdx.x * V;
-        for (; i + 256 * V < whole; i += 512 * V) {
-            Vec16<T> u = ld_vec_stream(x + i), w = ld_vec_stream(x + i + 256 * V);
+        for (; i + kBNT * V < whole; i += 2 * kBNT * V) {
+            Vec16<T> u = ld_vec_stream(x + i), w = ld_vec_stream(x + i + kBNT * V);
 #pragma unroll
             for (int k = 0; k < V; ++k) {
                 u.v[k] = one(u.v[k]);
                 w.v[k] = one(w.v[k]);
             }
             st_vec(xb + i, u);
-            st_vec(xb + i + 256 * V, w);
+            st_vec(xb + i + kBNT * V, w);
         }
         if (i < whole) {
             Vec16<T> u = ld_vec_stream(x + i);
@@ -213,7 +225,7 @@ __device__ void prod_map_tile(const adpar_batch_segment& sg, char* st, const Sta
         return;
     }
     // a zero among the elements: its own adjoint (when it is the only one), 0 elsewhere
-    for (int64_t i = lo + threadIdx.x; i < hi; i += 256)
+    for (int64_t i = lo + threadIdx.x; i < hi; i += kBNT)
         xb[i] = (f.nz == 1 && i == f.first && yb != 0.0) ? (T)ldexp_clamped(kq, f.e + ye) : T(0);
 }
 
@@ -248,13 +260,14 @@ __global__ void batch_init_kernel(char* ws, int64_t bytes) {
 }
 
 template <int RT>
-__global__ void __launch_bounds__(256) batch_kernel(const char* plan, char* ws) {
+__global__ void __launch_bounds__(kBNT, 4) batch_kernel(const char* plan, char* ws) {
     extern __shared__ __align__(16) unsigned char s_dyn[];  // kBRunSmem: the scan tiles' arrays
     const BatchPlanHeader* H = reinterpret_cast<const BatchPlanHeader*>(plan);
     const adpar_batch_segment* segs = reinterpret_cast<const adpar_batch_segment*>(plan + H->seg_off);
     const SegMeta* meta = reinterpret_cast<const SegMeta*>(plan + H->meta_off);
     WsHeader* hdr = reinterpret_cast<WsHeader*>(ws);
     const int64_t nseg = H->nseg, total = H->total_items;
+    // meta[nseg] closes the last segment: its item_base is where B(nseg - 1) begins
     __shared__ uint32_t s_item;
     __shared__ int s_stop;
     __shared__ int64_t s_seg;
@@ -262,7 +275,7 @@ __global__ void __launch_bounds__(256) batch_kernel(const char* plan, char* ws) 
     // next item's segment is found from there (usually the same segment: no
     // load at all; else a galloping search forward), instead of a binary
     // search of 12 dependent loads per item
-    int64_t seg = 0, seg_next = nseg > 1 ? meta[1].item_base : INT64_MAX;
+    int64_t seg = 0, seg_next = meta[1].item_base;
     while (true) {
         __syncthreads();  // consecutive items reuse the static shared memory
         if (threadIdx.x == 0) {
@@ -270,53 +283,50 @@ __global__ void __launch_bounds__(256) batch_kernel(const char* plan, char* ws) 
             s_stop = ((int64_t)s_item >= total) || gave_up(hdr);
             const int64_t q = s_item;
             if (!s_stop && q >= seg_next) {
-                // the last s with item_base <= q lies in (seg, nseg)
+                // the last s with item_base <= q lies in (seg, nseg]
                 int64_t lo = seg + 1, step = 1;
-                while (lo + step < nseg && meta[lo + step].item_base <= q) {
+                while (lo + step <= nseg && meta[lo + step].item_base <= q) {
                     lo += step;
                     step <<= 1;
                 }
-                int64_t hi = std::min<int64_t>(nseg - 1, lo + step - 1);
+                int64_t hi = std::min<int64_t>(nseg, lo + step - 1);
                 while (lo < hi) {
                     const int64_t mid = (lo + hi + 1) >> 1;
                     if (meta[mid].item_base <= q) lo = mid;
                     else hi = mid - 1;
                 }
                 seg = lo;
-                seg_next = seg + 1 < nseg ? meta[seg + 1].item_base : INT64_MAX;
+                seg_next = seg + 1 <= nseg ? meta[seg + 1].item_base : INT64_MAX;
             }
             s_seg = seg;
         }
         __syncthreads();
         if (s_stop) break;
-        const int64_t q = s_item;
-        const int64_t lo = s_seg;
-        const SegMeta m = meta[lo];
+        // block lo of the numbering: A(lo), then B(lo - 1)
+        int64_t lo = s_seg;
+        int64_t j = (int64_t)s_item - meta[lo].item_base;
+        SegMeta m = meta[lo];
+        const bool part_b = j >= (int64_t)m.red_tiles + m.scan_tiles;  // (meta[nseg] has no tiles)
+        if (part_b) {
+            j -= (int64_t)m.red_tiles + m.scan_tiles;
+            m = meta[--lo];
+        }
         const adpar_batch_segment sg = segs[lo];
         const StateLayout L = state_layout(sg.dtype, m.red_tiles, m.scan_tiles);
         char* st = ws + m.state_off;
-        int64_t j = q - m.item_base;
         const bool f64 = sg.dtype == ADPAR_F64;
-        if (j < m.red_tiles) {
+        if (!part_b && j < m.red_tiles) {
             if (f64) prod_reduce_tile<double>(sg, st, L, m.red_tiles, (int)j, RT, hdr);
             else prod_reduce_tile<float>(sg, st, L, m.red_tiles, (int)j, RT, hdr);
-            continue;
+        } else if (!part_b || j < m.scan_tiles) {
+            const int64_t k = part_b ? j : j - m.red_tiles;
+            if (f64) linrec_tile<double>(sg, st, L, m.scan_tiles, k, part_b, s_dyn, hdr);
+            else linrec_tile<float>(sg, st, L, m.scan_tiles, k, part_b, s_dyn, hdr);
+        } else {
+            j -= m.scan_tiles;
+            if (f64) prod_map_tile<double>(sg, st, L, (int)j, RT, hdr);
+            else prod_map_tile<float>(sg, st, L, (int)j, RT, hdr);
         }
-        j -= m.red_tiles;
-        if (j < m.scan_tiles) {
-            if (f64) linrec_tile<double>(sg, st, L, m.scan_tiles, j, false, s_dyn, hdr);
-            else linrec_tile<float>(sg, st, L, m.scan_tiles, j, false, s_dyn, hdr);
-            continue;
-        }
-        j -= m.scan_tiles;
-        if (j < m.scan_tiles) {
-            if (f64) linrec_tile<double>(sg, st, L, m.scan_tiles, j, true, s_dyn, hdr);
-            else linrec_tile<float>(sg, st, L, m.scan_tiles, j, true, s_dyn, hdr);
-            continue;
-        }
-        j -= m.scan_tiles;
-        if (f64) prod_map_tile<double>(sg, st, L, (int)j, RT, hdr);
-        else prod_map_tile<float>(sg, st, L, (int)j, RT, hdr);
     }
 }
 
@@ -332,7 +342,7 @@ BatchKernel kernel_of(int v) {
 
 size_t plan_bytes(int64_t nseg) {
     return round_up(sizeof(BatchPlanHeader), 64) + round_up((size_t)nseg * sizeof(adpar_batch_segment), 64) +
-           round_up((size_t)nseg * sizeof(SegMeta), 64);
+           round_up((size_t)(nseg + 1) * sizeof(SegMeta), 64);
 }
 
 }  // namespace
@@ -397,9 +407,12 @@ extern "C" int adpar_batch_plan(const adpar_batch_segment* segs, int nseg, const
         M[q].red_tiles = (int32_t)red;
         M[q].scan_tiles = (int32_t)scan;
         M[q].state_off = state;
-        items += 2 * red + 2 * scan;
+        items += red + scan;                                          // A(q)
+        if (q > 0) items += M[q - 1].red_tiles + (int64_t)M[q - 1].scan_tiles;  // B(q - 1)
         state += state_layout(g.dtype, (int)red, (int)scan).total;
     }
+    M[nseg].item_base = items;  // B(nseg - 1) alone
+    if (nseg > 0) items += M[nseg - 1].red_tiles + (int64_t)M[nseg - 1].scan_tiles;
     if (items > (int64_t)UINT32_MAX - ((int64_t)1 << 20)) return ADPAR_ERR_UNSUPPORTED;  // 32-bit tickets
     H->total_items = items;
     H->ws_bytes = (int64_t)round_up((size_t)state, 256);
@@ -430,8 +443,9 @@ extern "C" int adpar_vjp_batch(const void* plan_host, const void* plan_dev, void
             return ADPAR_ERR_CUDA;
         configured[dev][H->variant] = true;
     }
-    const int64_t grid = std::min<int64_t>((int64_t)sms * H->ctas_per_sm, H->total_items);
-    kernel_of(H->variant)<<<(unsigned)std::max<int64_t>(1, grid), 256, kBRunSmem, s>>>(
+    // ctas_per_sm counts blocks of 256 threads: twice as many of 128
+    const int64_t grid = std::min<int64_t>((int64_t)sms * H->ctas_per_sm * 2, H->total_items);
+    kernel_of(H->variant)<<<(unsigned)std::max<int64_t>(1, grid), kBNT, kBRunSmem, s>>>(
         static_cast<const char*>(plan_dev), static_cast<char*>(work));
     return cudaGetLastError() == cudaSuccess ? ADPAR_OK : ADPAR_ERR_CUDA;
 }

@@ -1,8 +1,11 @@
 // Linear-recurrence scan VJP tiles of the batched launch, on per-thread
 // runs (the rule and the two passes of scan_runs.cuh, Sec. 5.2), for
-// segments of any length inside one persistent kernel of 256 threads.
+// segments of any length inside one persistent kernel of 128-thread blocks.
 //
-// A tile is kBNT = 256 runs (one per thread) of one 128-byte row each.
+// A tile is kBNT = 128 runs (one per thread) of one 128-byte row each: 48 KB of
+// shared memory and 128 registers a thread let four tiles reside per SM, whose
+// loads, look-backs and FP64 folds overlap (tiles of 256 runs, two per SM, left
+// the FP64 pipe at 26%).
 //   forward tile t: folds its runs, scans them, looks back over the
 //     segment's earlier tiles for its exclusive prefix, and stores every
 //     run's exclusive carry (from the segment's start) and product of a;
@@ -20,13 +23,13 @@
 
 namespace adpar {
 
-constexpr int kBNT = 256;              // runs (threads) per batch tile
-constexpr int kBArr = kBNT * 128;      // one array's tile in bytes (32 KB)
+constexpr int kBNT = 128;              // runs (threads) per batch tile
+constexpr int kBArr = kBNT * 128;      // one array's tile in bytes (16 KB)
 constexpr int kBRunSmem = 3 * kBArr;   // shared memory of a reverse tile
 
 template <class T>
 constexpr int brun_tile() {
-    return kBNT * RunCfg<T>::V;  // elements per tile: 4096 FP64, 8192 FP32
+    return kBNT * RunCfg<T>::V;  // elements per tile: 2048 FP64, 4096 FP32
 }
 
 // Thread 0 asks L2 for elements [lo, hi) of p (the whole 16-byte units):
