@@ -351,15 +351,28 @@ __device__ __forceinline__ void prod_adjoint_body(const ReduceArgs& A, const Pro
         if (i < A.n) abar[i] = A.accumulate ? abar[i] + one(a[i]) : one(a[i]);
         return;
     }
-    for (int64_t i = t0; i < A.n; i += stride) {
-        double c = 0.0;
-        if (yb != 0.0) {
-            if (st.nz == 1 && i == st.first) {
-                c = ldexp_clamped(st.m * ym, st.e + ye);
-            }
+    // zeros among the elements (or ybar = 0): 0, and the only zero's own adjoint
+    const int64_t at = st.nz == 1 && yb != 0.0 ? st.first : -1;
+    auto value = [&](int64_t i) -> T { return i == at ? (T)ldexp_clamped(kq, st.e + ye) : T(0); };
+    constexpr int V = Vec16<T>::N;
+    const int64_t nv = A.n / V;
+    for (int64_t v = t0; v < nv; v += stride) {
+        Vec16<T> o;
+#pragma unroll
+        for (int k = 0; k < V; ++k) o.v[k] = T(0);
+        if (at / V == v && at >= 0) {
+#pragma unroll
+            for (int k = 0; k < V; ++k) o.v[k] = value(v * V + k);
         }
-        abar[i] = A.accumulate ? (T)((double)abar[i] + c) : (T)c;
+        T* p = abar + v * V;
+        if (A.accumulate) {
+#pragma unroll
+            for (int k = 0; k < V; ++k) o.v[k] += p[k];
+        }
+        st_vec(p, o);
     }
+    const int64_t i = nv * V + t0;
+    if (i < A.n) abar[i] = A.accumulate ? abar[i] + value(i) : value(i);
 }
 
 template <class T>
@@ -373,12 +386,12 @@ __global__ void __launch_bounds__(kRedBlock, 4) prod_adjoint_kernel(ReduceArgs A
 // block reduces its share, the blocks read each other's states through
 // distributed shared memory (a hardware barrier of the cluster instead of a
 // global counter that an earlier launch must clear), and every block maps its
-// share with the same total.  65536 FP64 values: 11 us on the device against 17 in
-// three launches (and their gaps), 29.5 against 35.6 us per call from Python; at 2 MB
-// 28 against 32, at 4 MB 45 against 32.
+// share with the same total.  65536 FP64 values: 10 us on the device against 17 in
+// three launches and their gaps (14 against 18 us per call from Python, on a slow
+// host); at 1 MB 18 against 18, at 2 MB 26 against 18.
 constexpr int kClusterBlocks = 8;
 constexpr int kClusterThreads = 1024;
-constexpr int64_t kClusterBytes = int64_t(2) << 20;
+constexpr int64_t kClusterBytes = int64_t(1) << 20;
 
 __device__ __forceinline__ void cluster_sync() {
     asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
@@ -434,12 +447,10 @@ __global__ void __cluster_dims__(kClusterBlocks, 1, 1) __launch_bounds__(kCluste
         S q = (int)threadIdx.x < kClusterBlocks ? ld_cluster(&s_block, threadIdx.x) : S::id();
 #pragma unroll
         for (int off = kClusterBlocks / 2; off > 0; off >>= 1) q = S::comb(q, shfl_down_s(q, off));
-        if (threadIdx.x == 0) {
-            s_total = q.to_state();
-            if (blockIdx.x == 0) prod_results<T>(A, s_total);
-        }
+        if (threadIdx.x == 0) s_total = q.to_state();
     }
     __syncthreads();
+    if (t0 == 32) prod_results<T>(A, s_total);  // beside the map
     if (!A.primal_only) prod_adjoint_body<T>(A, s_total, t0, stride);
     cluster_sync();  // no block leaves while another may read its state
 }

@@ -77,13 +77,13 @@ def test_sizes(dt, rel, n, accumulate):
         assert np.all(np.abs(got - ref) <= np.abs(ref) * rel * (1 + n * 2.0 ** -14 * (dt == np.float64)))
 
 
-# one cluster of 8 x 1024 threads up to 2 MB, three launches beyond
+# one cluster of 8 x 1024 threads up to 1 MB, three launches beyond
 @pytest.mark.parametrize("dt", [np.float64, np.float32])
 @pytest.mark.parametrize("over", [-1, 0, 1])
 @pytest.mark.parametrize("zeros", [0, 1, 2])
 def test_one_cluster_boundary(dt, over, zeros):
     from paper_2202_10297_gb300 import adpar as A
-    n = (2 << 20) // np.dtype(dt).itemsize + over
+    n = (1 << 20) // np.dtype(dt).itemsize + over
     g = np.random.default_rng(n + zeros)
     a = np.exp(g.uniform(-2.0 ** -10, 2.0 ** -10, n)).astype(dt)
     pos = np.sort(g.choice(n, zeros, replace=False))
