@@ -18,9 +18,8 @@
 //              accumulators (2 x 256 columns).  The distance is
 //              |x|^2 - 2 acc_k, so the argmin is the argmax of acc.
 //   warps 2-17 epilogue, two groups of 8 warps taking alternate tiles (group
-//              p reads accumulator p and synchronises on its own named
-//              barrier), tiles handed out by a global ticket through the
-//              producer.  In a group, two threads per row (warp w reads the
+//              p reads accumulator p), tiles handed out by a global ticket
+//              through the producer.  In a group, two threads per row (warp w reads the
 //              TMEM lanes of quarter w % 4, and every other 32-column chunk):
 //              a tcgen05.ld.red pass (the load's own max reduction, sm_103a)
 //              for the largest acc_k; the row's maximum from its two
@@ -109,24 +108,41 @@ __device__ __forceinline__ float sw_elem(const float* tile, int r, int j) {
 // squares of its 8 coordinates (x0, x1: the row's chunks 2 g, 2 g + 1), then
 // two butterfly steps add the partial sums, so that the four lanes hold the
 // same value.  All lanes of the warp call it.
-__device__ __forceinline__ float cand_dist_f32(const float4& x0, const float4& x1, const float* sC, int kc, int g) {
+// Two coordinates per instruction (packed FP32 fused multiply-adds, each
+// lane rounded as a scalar one): x - c as c * (-1) + x, then its square.
+__device__ __forceinline__ unsigned long long fma_f32x2(unsigned long long a, unsigned long long b,
+                                                        unsigned long long c) {
+    unsigned long long d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+__device__ __forceinline__ unsigned long long add_f32x2(unsigned long long a, unsigned long long b) {
+    unsigned long long d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ unsigned long long pack_f32x2(uint32_t lo, uint32_t hi) {
+    unsigned long long d;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "r"(lo), "r"(hi));
+    return d;
+}
+__device__ __forceinline__ float cand_dist_f32(const ulonglong2& x0, const ulonglong2& x1, const float* sC, int kc,
+                                               int g) {
     const float* crow = sC + kc * KM_D;
-    const float4 c0 = *reinterpret_cast<const float4*>(crow + (((2 * g) ^ (kc & 7)) * 4));
-    const float4 c1 = *reinterpret_cast<const float4*>(crow + (((2 * g + 1) ^ (kc & 7)) * 4));
-    // two chains of four (chunk 2 g, chunk 2 g + 1), then their sum
-    float d, s = 0.f, u = 0.f;
-    d = x0.x - c0.x; s = fmaf(d, d, s);
-    d = x1.x - c1.x; u = fmaf(d, d, u);
-    d = x0.y - c0.y; s = fmaf(d, d, s);
-    d = x1.y - c1.y; u = fmaf(d, d, u);
-    d = x0.z - c0.z; s = fmaf(d, d, s);
-    d = x1.z - c1.z; u = fmaf(d, d, u);
-    d = x0.w - c0.w; s = fmaf(d, d, s);
-    d = x1.w - c1.w; u = fmaf(d, d, u);
-    s += u;
-    s += __shfl_xor_sync(0xffffffffu, s, 1);
-    s += __shfl_xor_sync(0xffffffffu, s, 2);
-    return s;
+    const ulonglong2 c0 = *reinterpret_cast<const ulonglong2*>(crow + (((2 * g) ^ (kc & 7)) * 4));
+    const ulonglong2 c1 = *reinterpret_cast<const ulonglong2*>(crow + (((2 * g + 1) ^ (kc & 7)) * 4));
+    constexpr unsigned long long kNeg1 = 0xbf800000bf800000ull;
+    // two chains of two pairs, then their sum
+    unsigned long long d, s, u;
+    d = fma_f32x2(c0.x, kNeg1, x0.x); s = fma_f32x2(d, d, 0ull);
+    d = fma_f32x2(c1.x, kNeg1, x1.x); u = fma_f32x2(d, d, 0ull);
+    d = fma_f32x2(c0.y, kNeg1, x0.y); s = fma_f32x2(d, d, s);
+    d = fma_f32x2(c1.y, kNeg1, x1.y); u = fma_f32x2(d, d, u);
+    s = add_f32x2(s, u);
+    float r = __uint_as_float((uint32_t)s) + __uint_as_float((uint32_t)(s >> 32));
+    r += __shfl_xor_sync(0xffffffffu, r, 1);
+    r += __shfl_xor_sync(0xffffffffu, r, 2);
+    return r;
 }
 
 // the oracle's FP64 arithmetic: s += (x - c)^2 with no fused multiply-add
@@ -148,14 +164,16 @@ __global__ void km_empty_kernel(float* loss_out, float* Cbar, int kd, int accumu
         for (int q = t; q < kd; q += gridDim.x * blockDim.x) Cbar[q] = 0.f;
 }
 
-// The 16 epilogue warps (warps 2-17) form two groups of 8 (256 threads)
-// that take alternate tiles, group p synchronising on named barrier 1 + p.
-// epi_any is a barrier that also ORs a predicate over the group, so a
+// The 16 epilogue warps (warps 2-17) form two groups of 8 that take alternate
+// tiles; in a group, the two warps that read a quarter of the rows exchange all
+// they need between themselves, on a named barrier of their own (64 threads).
+// pair_any is that barrier with the OR of a predicate over the pair, so a
 // decision to stop is taken by all of its threads together.
-__device__ __forceinline__ void epi_sync(int pg) {
-    asm volatile("bar.sync %0, %1;" ::"r"(1 + pg), "r"(KM_PG_THREADS) : "memory");
+constexpr int KM_PAIR_THREADS = 64;
+__device__ __forceinline__ void pair_sync(int id) {
+    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(KM_PAIR_THREADS) : "memory");
 }
-__device__ __forceinline__ bool epi_any(int pg, bool p) {
+__device__ __forceinline__ bool pair_any(int id, bool p) {
     uint32_t r;
     asm volatile(
         "{\n\t.reg .pred q, o;\n\t"
@@ -163,7 +181,7 @@ __device__ __forceinline__ bool epi_any(int pg, bool p) {
         "bar.red.or.pred o, %2, %3, q;\n\t"
         "selp.u32 %0, 1, 0, o;\n\t}"
         : "=r"(r)
-        : "r"((uint32_t)p), "r"(1 + pg), "r"(KM_PG_THREADS)
+        : "r"((uint32_t)p), "r"(id), "r"(KM_PAIR_THREADS)
         : "memory");
     return r != 0;
 }
@@ -219,7 +237,7 @@ __global__ void __launch_bounds__(KM_THREADS, 1)
         }
         for (int b = 0; b < 2; ++b) {
             tc::mbar_init(&t_full[b], 1);
-            tc::mbar_init(&t_empty[b], 1);  // one arrival after the epilogue barrier
+            tc::mbar_init(&t_empty[b], KM_PG_THREADS / 32);  // one arrival per warp of a group
         }
         tc::mbar_init(c_bar, 1);
         *s_abort = 0;
@@ -333,6 +351,7 @@ __global__ void __launch_bounds__(KM_THREADS, 1)
         const int r = quarter * 32 + lane;  // row of the tile == TMEM lane
         const uint32_t lane_base = (uint32_t)(quarter * 32) << 16;
         const int nq = k / 32;
+        const int pair_id = 1 + pg * 4 + quarter;
         float* g_max = s_max + pg * KM_TPR * KM_TILE;
         float* g_xn = s_xn + pg * KM_TPR * KM_TILE;
         int* g_ncnt = s_ncnt + pg * KM_TILE * KM_TPR;
@@ -384,7 +403,7 @@ __global__ void __launch_bounds__(KM_THREADS, 1)
                 m1 = fmaxf(m1, cm);
             }
             g_max[grp * KM_TILE + r] = m1;
-            if (epi_any(pg, !ok)) break;  // every thread of the group leaves together
+            if (pair_any(pair_id, !ok)) break;  // both warps of the pair leave together
             float amax = g_max[r], xn2 = g_xn[r];
 #pragma unroll
             for (int g = 1; g < KM_TPR; ++g) {
@@ -399,6 +418,7 @@ __global__ void __launch_bounds__(KM_THREADS, 1)
             // computed maximum, and tol is 4x that bound
             const float tol = 8.0e-3f * xn * cmax + 1.0e-5f * (cmax * cmax + xn * cmax) + 1e-20f;
             const float thr = amax - tol;
+            const unsigned long long nthr = pack_f32x2(__float_as_uint(-thr), __float_as_uint(-thr));
             // pass 2: candidates, every column within tol of the row's maximum
             // (this thread's first KM_SLOTS in its own slots; a count above
             // KM_SLOTS sends the row to the all-centroids path)
@@ -409,11 +429,17 @@ __global__ void __launch_bounds__(KM_THREADS, 1)
                 __syncwarp();
                 tc::tmem_ld32(tb + (uint32_t)(q * 32), va);
                 tc::tmem_ld_wait();
-                // four independent OR chains (one long chain waits on itself)
-                uint32_t mk[4] = {0u, 0u, 0u, 0u};
+                // bit j = (va[j] >= thr) from the sign of va[j] - thr: packed
+                // subtractions, then one funnel shift per value collects the signs,
+                // in four independent chains
+                uint32_t sg[4] = {0u, 0u, 0u, 0u};
 #pragma unroll
-                for (int j = 0; j < 32; ++j) mk[j & 3] |= (__uint_as_float(va[j]) >= thr ? 1u : 0u) << j;
-                uint32_t mask = (mk[0] | mk[1]) | (mk[2] | mk[3]);
+                for (int j = 30; j >= 0; j -= 2) {
+                    const unsigned long long d = add_f32x2(pack_f32x2(va[j], va[j + 1]), nthr);
+                    sg[j >> 3] = __funnelshift_l((uint32_t)(d >> 32), sg[j >> 3], 1);
+                    sg[j >> 3] = __funnelshift_l((uint32_t)d, sg[j >> 3], 1);
+                }
+                uint32_t mask = ~(sg[0] | (sg[1] << 8) | (sg[2] << 16) | (sg[3] << 24));
                 while (mask) {
                     const int j = __ffs(mask) - 1;
                     mask &= mask - 1;
@@ -422,20 +448,22 @@ __global__ void __launch_bounds__(KM_THREADS, 1)
                 }
             }
             g_ncnt[r * KM_TPR + grp] = ncnt;
-            // every thread of the group has read the accumulator past this barrier
+            // this warp has read the accumulator; the pair's lists are complete
+            // past its barrier
             tc::fence_before_sync();
-            epi_sync(pg);
-            if (gw == 0 && lane == 0) tc::mbar_arrive(&t_empty[b]);
+            __syncwarp();
+            if (lane == 0) tc::mbar_arrive(&t_empty[b]);
+            pair_sync(pair_id);
 
-            // certification, loss and row sums: warp gw takes rows 16 gw ..
-            // 16 gw + 15, 8 at a time, four adjacent lanes per row, lane g of
-            // a row the coordinates 8 g .. 8 g + 7
+            // certification, loss and row sums: each warp of the pair takes 16
+            // of its quarter's rows, 8 at a time, four adjacent lanes per row,
+            // lane g of a row the coordinates 8 g .. 8 g + 7
 #pragma unroll 1
             for (int rd = 0; rd < 2; ++rd) {
-                const int rc = gw * 16 + rd * 8 + (lane >> 2), g = lane & 3;
+                const int rc = quarter * 32 + grp * 16 + rd * 8 + (lane >> 2), g = lane & 3;
                 const float* xrow = xt + rc * KM_D;
-                const float4 x0 = *reinterpret_cast<const float4*>(xrow + (((2 * g) ^ (rc & 7)) * 4));
-                const float4 x1 = *reinterpret_cast<const float4*>(xrow + (((2 * g + 1) ^ (rc & 7)) * 4));
+                const ulonglong2 x0 = *reinterpret_cast<const ulonglong2*>(xrow + (((2 * g) ^ (rc & 7)) * 4));
+                const ulonglong2 x1 = *reinterpret_cast<const ulonglong2*>(xrow + (((2 * g + 1) ^ (rc & 7)) * 4));
                 // the row's candidates: scanning thread 0's first min(count,
                 // KM_SLOTS) slots, then thread 1's; a count above KM_SLOTS
                 // makes every centroid a candidate
@@ -513,14 +541,12 @@ __global__ void __launch_bounds__(KM_THREADS, 1)
                         // (a row at a time with lanes = its 32 coordinates,
                         // conflict-free, measured slower: 0.225 -> 0.250 ms)
                         float* srow = s_sum + best * KM_SUM_LD + 8 * g;
-                        atomicAdd(srow + 0, x0.x);
-                        atomicAdd(srow + 1, x0.y);
-                        atomicAdd(srow + 2, x0.z);
-                        atomicAdd(srow + 3, x0.w);
-                        atomicAdd(srow + 4, x1.x);
-                        atomicAdd(srow + 5, x1.y);
-                        atomicAdd(srow + 6, x1.z);
-                        atomicAdd(srow + 7, x1.w);
+                        const unsigned long long xs[4] = {x0.x, x0.y, x1.x, x1.y};
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) {
+                            atomicAdd(srow + 2 * q, __uint_as_float((uint32_t)xs[q]));
+                            atomicAdd(srow + 2 * q + 1, __uint_as_float((uint32_t)(xs[q] >> 32)));
+                        }
                         if (g == 0) atomicAdd(&s_cnt[best], 1.f);
                     }
                 }
