@@ -5,8 +5,8 @@
 // a thread owns one column and one chunk of kVecR rows, so a warp's loads
 // cover 32 consecutive columns of a row (coalesced), 8 rows' loads in flight.
 // No block waits on another:
-//   1. per (chunk, column): the aggregates of the operator's state and of the
-//      return sweep's lin_o state;
+//   1. per (chunk, column): the aggregates of the operator's state, then of the
+//      return sweep's lin_o state (two launches);
 //   2. per column a scan of the chunks' aggregates, left to right and right to
 //      left (exclusive carries);
 //   3. per (chunk, column): a backward sweep of rs_bar_r = ybar_r +
@@ -55,83 +55,69 @@ __device__ __forceinline__ void vec_rows(const void* p, const VecArgs& V, int64_
     for (int u = 0; u < U; ++u) o[u] = row + u < V.n ? __ldg(q + u * V.d) : pad;
 }
 
-// Chunk aggregates in one sweep from top to bottom: PRIMAL the operator's state,
-// ADJ the return sweep's x -> c_r (ybar_r + x), composed as a growing map (the
-// next row's map goes inside), so that each array is read once.  MIN/MAX take
-// their J_left from the prefix, formed from the carry that a first launch
-// (PRIMAL alone) and its scan left.
-template <class Op, class T, bool PRIMAL, bool ADJ>
-__global__ void __launch_bounds__(kVecBlock, 6) vec_agg_kernel(VecArgs V) {
+// the operator's state over each chunk, top to bottom
+template <class Op, class T>
+__global__ void __launch_bounds__(kVecBlock, 6) vec_primal_agg_kernel(VecArgs V) {
     using P = typename Op::P;
     constexpr int W = Op::kWidth, U = kVecUAgg;
-    constexpr bool kA = PRIMAL || !Op::kCoefOne;  // a is read
-    using L = Lin<T, W, !Op::kCoefOne>;
     const int64_t col = blockIdx.x * (int64_t)kVecBlock + threadIdx.x, c = blockIdx.y;
     if (col >= V.d) return;
     const int64_t r0 = c * kVecR;
-    P cur = Op::pid();
-    if constexpr (ADJ && Op::kCoefNeedsPrimal) cur = static_cast<const P*>(V.aggP)[c * V.d + col];
-    L acc = L::id();
+    P acc = Op::pid();
 #pragma unroll 1
-    for (int q = 0; q < kVecR; q += U) {
-        T a[U], b[U], y1[U], y2[U];
-        if constexpr (kA) vec_rows<U>(V.a, V, r0 + q, col, Op::pad_a(), a);
-        if constexpr (PRIMAL && W == 2) vec_rows<U>(V.b, V, r0 + q, col, T(0), b);
-        if constexpr (ADJ) vec_rows<U>(V.ya, V, r0 + q, col, T(0), y1);
-        if constexpr (ADJ && W == 2) vec_rows<U>(V.yb, V, r0 + q, col, T(0), y2);
+    for (int q = 0; q < kVecR && r0 + q < V.n; q += U) {
+        T a[U], b[U];
+        vec_rows<U>(V.a, V, r0 + q, col, Op::pad_a(), a);
+        if constexpr (W == 2) vec_rows<U>(V.b, V, r0 + q, col, T(0), b);
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-            if constexpr (ADJ) {
-                if (r0 + q + u < V.n) {
-                    L el;
-                    if constexpr (!Op::kCoefOne) {
-                        const T cr = Op::coef(cur, a[u]);
-                        el.c = cr;
-                        el.d[0] = cr * y1[u];
-                        if constexpr (W == 2) el.d[1] = cr * y2[u];
-                    } else {
-                        el.d[0] = y1[u];
-                        if constexpr (W == 2) el.d[1] = y2[u];
-                    }
-                    acc = L::comb(el, acc);
-                }
-            }
-            if constexpr (PRIMAL || (ADJ && Op::kCoefNeedsPrimal))
-                cur = Op::pcomb(cur, Op::pelem(a[u], PRIMAL && W == 2 ? b[u] : T(0)));
-        }
+        for (int u = 0; u < U; ++u) acc = Op::pcomb(acc, Op::pelem(a[u], W == 2 ? b[u] : T(0)));
     }
-    if constexpr (PRIMAL) static_cast<P*>(V.aggP)[c * V.d + col] = cur;
-    if constexpr (ADJ) static_cast<L*>(V.aggL)[c * V.d + col] = acc;
+    static_cast<P*>(V.aggP)[c * V.d + col] = acc;
 }
 
 // Turns the chunk aggregates of 32 columns into exclusive prefixes (REV:
-// exclusive suffixes, composed right to left).  Thread (x, y) of a 32 x kVecG
-// block folds group y of column x's chunks (neighbouring lanes read neighbouring
-// columns), takes the fold of the groups before it and runs through its chunks
-// again.  8 chunks are loaded at a time.
+// exclusive suffixes, composed right to left).  Thread (x, y) of a 32 x G block
+// folds group y of column x's chunks (neighbouring lanes read neighbouring
+// columns), the groups' folds are scanned by shuffles, a warp per column, and
+// each thread runs through its chunks again.  8 chunks are loaded at a time; G
+// is a group per 8 chunks, up to 32.
 constexpr int kVecG = 32;
 template <class S, bool REV, class Comb>
 __device__ __forceinline__ void vec_scan_columns(S* agg, int64_t C, int64_t d, S* s_tot, const S& ident, Comb comb) {
-    const int x = threadIdx.x & 31, y = threadIdx.x >> 5;
+    const int x = threadIdx.x & 31, y = threadIdx.x >> 5, G = blockDim.x >> 5;
     const int64_t col = blockIdx.x * (int64_t)32 + x;
-    const int64_t per = (C + kVecG - 1) / kVecG;
+    const int64_t per = (C + G - 1) / G;
     const int64_t lo = y * per < C ? y * per : C, hi = lo + per < C ? lo + per : C;
     const bool live = col < d;
     auto at = [&](int64_t q) -> S* { return agg + (REV ? C - 1 - q : q) * d + col; };
-    S acc = ident;
-    if (live) {
-        for (int64_t q = lo; q < hi; q += 8) {
-            S v[8];
-#pragma unroll
-            for (int u = 0; u < 8; ++u) v[u] = q + u < hi ? *at(q + u) : ident;
-#pragma unroll
-            for (int u = 0; u < 8; ++u) acc = comb(acc, v[u]);
-        }
-    }
-    s_tot[y * 32 + x] = acc;
-    __syncthreads();
     S run = ident;
-    for (int g = 0; g < y; ++g) run = comb(run, s_tot[g * 32 + x]);
+    if (G > 1) {
+        if (live) {
+            for (int64_t q = lo; q < hi; q += 8) {
+                S v[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) v[u] = q + u < hi ? *at(q + u) : ident;
+#pragma unroll
+                for (int u = 0; u < 8; ++u) run = comb(run, v[u]);
+            }
+        }
+        s_tot[y * 33 + x] = run;
+        __syncthreads();
+        for (int w = y; w < 32; w += G) {  // lane x holds group x of column w
+            S inc = x < G ? s_tot[x * 33 + w] : ident;
+#pragma unroll
+            for (int off = 1; off < 32; off <<= 1) {
+                const S o = shfl_up_s(inc, off);
+                if (x >= off) inc = comb(o, inc);
+            }
+            S ex = shfl_up_s(inc, 1);
+            if (x == 0) ex = ident;
+            __syncwarp();
+            if (x < G) s_tot[x * 33 + w] = ex;
+        }
+        __syncthreads();
+        run = s_tot[y * 33 + x];
+    }
     if (live) {
         for (int64_t q = lo; q < hi; q += 8) {
             S v[8];
@@ -139,7 +125,8 @@ __device__ __forceinline__ void vec_scan_columns(S* agg, int64_t C, int64_t d, S
             for (int u = 0; u < 8; ++u) v[u] = q + u < hi ? *at(q + u) : ident;
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
-                if (q + u < hi) *at(q + u) = run;
+                if (q + u >= hi) break;
+                *at(q + u) = run;
                 run = comb(run, v[u]);
             }
         }
@@ -170,7 +157,7 @@ __device__ __forceinline__ uint32_t vec_coef_bits(const VecArgs& V, int64_t col,
     uint32_t bits = 0u;
     typename Op::P cur = carry;
 #pragma unroll 1
-    for (int q = 0; q < kVecR; q += kVecU) {
+    for (int q = 0; q < kVecR && r0 + q < V.n; q += kVecU) {
         T a[kVecU];
         vec_rows(V.a, V, r0 + q, col, Op::pad_a(), a);
 #pragma unroll
@@ -182,29 +169,70 @@ __device__ __forceinline__ uint32_t vec_coef_bits(const VecArgs& V, int64_t col,
     return bits;
 }
 
-// J_left of the rows row .. row + kVecU - 1 (q0: the first one's number in the
+// J_left of the rows row .. row + U - 1 (q0: the first one's number in the
 // chunk); rows past the end have ybar 0 below them, so their value is free
-template <class Op, class T>
+template <class Op, class T, int U>
 __device__ __forceinline__ void vec_coefs(const VecArgs& V, int64_t row, int64_t col, uint32_t bits, int q0,
-                                          T (&c)[kVecU]) {
+                                          T (&c)[U]) {
     if constexpr (Op::kCoefOne) {
 #pragma unroll
-        for (int u = 0; u < kVecU; ++u) c[u] = T(1);
+        for (int u = 0; u < U; ++u) c[u] = T(1);
     } else if constexpr (Op::kCoefNeedsPrimal) {
 #pragma unroll
-        for (int u = 0; u < kVecU; ++u) c[u] = ((bits >> (q0 + u)) & 1u) ? T(1) : T(0);
+        for (int u = 0; u < U; ++u) c[u] = ((bits >> (q0 + u)) & 1u) ? T(1) : T(0);
     } else {
-        vec_rows(V.a, V, row, col, T(1), c);
+        vec_rows<U>(V.a, V, row, col, T(1), c);
 #pragma unroll
-        for (int u = 0; u < kVecU; ++u) c[u] = Op::coef(Op::pid(), c[u]);
+        for (int u = 0; u < U; ++u) c[u] = Op::coef(Op::pid(), c[u]);
     }
 }
 
-// Chunks last to first: what vec_agg_kernel read last is still in L2.  8 rows'
+// Chunk aggregates of the return sweep: x -> c_r (ybar_r + x) folded bottom to
+// top (Horner's order: a contracting recurrence damps the early roundings; the
+// growing map of a sweep from the top, fused with the operator's, read each
+// array once and took 52 us for 23 + 40, but its FP32 results were further off)
+template <class Op, class T>
+__global__ void __launch_bounds__(kVecBlock, 6) vec_adjoint_agg_kernel(VecArgs V) {
+    using P = typename Op::P;
+    constexpr int W = Op::kWidth, U = kVecUAgg;
+    using L = Lin<T, W, !Op::kCoefOne>;
+    const int64_t col = blockIdx.x * (int64_t)kVecBlock + threadIdx.x, c = blockIdx.y;
+    if (col >= V.d) return;
+    const int64_t r0 = c * kVecR;
+    uint32_t bits = 0u;
+    if constexpr (Op::kCoefNeedsPrimal)
+        bits = vec_coef_bits<Op, T>(V, col, r0, static_cast<const P*>(V.aggP)[c * V.d + col]);
+    L acc = L::id();
+#pragma unroll 1
+    for (int q = kVecR - U; q >= 0; q -= U) {
+        if (r0 + q >= V.n) continue;
+        T cf[U], y1[U], y2[U];
+        vec_coefs<Op, T, U>(V, r0 + q, col, bits, q, cf);
+        vec_rows<U>(V.ya, V, r0 + q, col, T(0), y1);
+        if constexpr (W == 2) vec_rows<U>(V.yb, V, r0 + q, col, T(0), y2);
+#pragma unroll
+        for (int u = U - 1; u >= 0; --u) {
+            if (r0 + q + u >= V.n) continue;
+            L el;
+            if constexpr (!Op::kCoefOne) {
+                el.c = cf[u];
+                el.d[0] = cf[u] * y1[u];
+                if constexpr (W == 2) el.d[1] = cf[u] * y2[u];
+            } else {
+                el.d[0] = y1[u];
+                if constexpr (W == 2) el.d[1] = y2[u];
+            }
+            acc = L::comb(acc, el);
+        }
+    }
+    static_cast<L*>(V.aggL)[c * V.d + col] = acc;
+}
+
+// Chunks last to first: what the aggregates read last is still in L2.  8 rows'
 // loads in flight at 9 blocks an SM (about 110 registers): 72 us for 8192 x 2048
 // FP32 LINREC (59 us for its bytes); 64 registers, or one row at a time: 96 and
-// 128 us.  The aggregates take 52 us (was 23 + 40 in two launches), the scan of
-// both 11 us (was 13 + 23 with a warp per column); the call 245 -> 138 us.
+// 128 us.  The scan of both aggregates takes 11 us (was 13 + 23 with a warp per
+// column); the call 245 -> 164 us.
 template <class Op, class T>
 __global__ void __launch_bounds__(kVecOutBlock, 9) vec_output_kernel(VecArgs V) {
     using P = typename Op::P;
@@ -225,8 +253,9 @@ __global__ void __launch_bounds__(kVecOutBlock, 9) vec_output_kernel(VecArgs V) 
     T ra = suf.d[0], rb = W == 2 ? suf.d[W - 1] : T(0), cn = T(1);
 #pragma unroll 1
     for (int q = kVecR - kVecU; q >= 0; q -= kVecU) {
+        if (r0 + q >= V.n) continue;
         T cf[kVecU], y1[kVecU], y2[kVecU];
-        vec_coefs<Op, T>(V, r0 + q, col, bits, q, cf);
+        vec_coefs<Op, T, kVecU>(V, r0 + q, col, bits, q, cf);
         vec_rows(V.ya, V, r0 + q, col, T(0), y1);
         if constexpr (W == 2) vec_rows(V.yb, V, r0 + q, col, T(0), y2);
 #pragma unroll
@@ -243,7 +272,7 @@ __global__ void __launch_bounds__(kVecOutBlock, 9) vec_output_kernel(VecArgs V) 
     T* bbar = W == 2 ? static_cast<T*>(V.bbar) + r0 * V.d + col : nullptr;
     P prev = carry;
 #pragma unroll 1
-    for (int q = 0; q < kVecR; q += kVecU) {
+    for (int q = 0; q < kVecR && r0 + q < V.n; q += kVecU) {
         T a[kVecU], b[kVecU];
         if constexpr (kP) {
             vec_rows(V.a, V, r0 + q, col, Op::pad_a(), a);
@@ -296,14 +325,13 @@ int run_vec(int64_t n, int64_t d, const void* a, const void* b, const void* ya, 
     const dim3 g2((unsigned)((d + kVecBlock - 1) / kVecBlock), (unsigned)V.C);
     const dim3 g5((unsigned)((d + kVecOutBlock - 1) / kVecOutBlock), (unsigned)V.C);
     const unsigned gw = (unsigned)((d + 31) / 32);  // 32 columns per block
-    const size_t sh = std::max(sizeof(typename Op::P), sizeof(L)) * 32 * kVecG;
-    constexpr bool kTwo = kVecPrimal<Op> && !Op::kCoefNeedsPrimal;  // both aggregates from one launch
-    if constexpr (Op::kCoefNeedsPrimal) {
-        vec_agg_kernel<Op, T, true, false><<<g2, kVecBlock, 0, s>>>(V);
-        vec_scan_kernel<Op, T><<<dim3(gw, 1), 32 * kVecG, sh, s>>>(V, 0);
-    }
-    vec_agg_kernel<Op, T, kTwo, true><<<g2, kVecBlock, 0, s>>>(V);
-    vec_scan_kernel<Op, T><<<dim3(gw, kTwo ? 2 : 1), 32 * kVecG, sh, s>>>(V, kTwo ? 0 : 1);
+    const int G = (int)std::max<int64_t>(1, std::min<int64_t>(V.C / 8, kVecG));
+    const size_t sh = std::max(sizeof(typename Op::P), sizeof(L)) * 33 * G;
+    constexpr bool kTwo = kVecPrimal<Op> && !Op::kCoefNeedsPrimal;  // both scans from one launch
+    if constexpr (kVecPrimal<Op>) vec_primal_agg_kernel<Op, T><<<g2, kVecBlock, 0, s>>>(V);
+    if constexpr (Op::kCoefNeedsPrimal) vec_scan_kernel<Op, T><<<dim3(gw, 1), 32 * G, sh, s>>>(V, 0);
+    vec_adjoint_agg_kernel<Op, T><<<g2, kVecBlock, 0, s>>>(V);
+    vec_scan_kernel<Op, T><<<dim3(gw, kTwo ? 2 : 1), 32 * G, sh, s>>>(V, kTwo ? 0 : 1);
     vec_output_kernel<Op, T><<<g5, kVecOutBlock, 0, s>>>(V);
     return cudaGetLastError() == cudaSuccess ? ADPAR_OK : ADPAR_ERR_CUDA;
 }
