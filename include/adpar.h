@@ -585,8 +585,9 @@ typedef struct {
 } adpar_batch_segment;
 
 /* Launch shape chosen by the autotuner: variant = compiled tile shapes
- * (0: 2048-element scan tiles, 8192-element product tiles; 1: 4096 /
- * 16384; 2: 1024 / 4096), ctas_per_sm = persistent blocks per SM (1..8),
+ * (product tiles of 8192, 16384 or 4096 elements for 0, 1, 2; the scan tiles
+ * are 128 runs of a 128-byte row in each), ctas_per_sm = persistent blocks per
+ * SM (1..8) in units of 256 threads (the kernel runs twice as many of 128),
  * order = 0 (as given) or 1 (longest segments first). */
 typedef struct {
     int32_t variant;
