@@ -268,8 +268,8 @@ __device__ __forceinline__ double recip_mantissa(double m) {
 // is below 2^-21, and K / m = K R (1 + eps + eps^2) up to eps^3 and the
 // 2^-52 resolution of eps: within 2^-50.1 of K / m with the final rounding
 // (2e7 mantissa pairs, edges among them, checked on the host).
-// Results outside the normal range leave by scale_pow2.  About 45 integer
-// instructions; with the one FP64 multiply and 64-bit Newton step that were
+// Results outside the normal range leave by scale_pow2.  About 100 instructions a
+// value in all, on the integer pipes; with the one FP64 multiply and 64-bit Newton step that were
 // here, the map over 2^26 values took 414 us, now 226 us with the loads four
 // vectors deep (158 us for its bytes); the reduction 275 us, now 102 us (79).
 struct QuotF64 {
