@@ -4,10 +4,10 @@
 // (number of zeros, lowest zero index, product of the nonzero elements).
 // The product of the nonzeros leaves every floating-point range on
 // realistic sizes (a product of 65536 values from U[0.5,1.5) is about
-// 1e-1287), so it is carried as  p = m * 2^e  with an FP64 mantissa m in
-// [0.5, 1) and a 64-bit exponent e.  The exponent split uses the bits of
-// the IEEE-754 representation (no FP64 arithmetic), so each element costs
-// one FP64 multiply.
+// 1e-1287), so it is carried as a mantissa and a 64-bit exponent: 64-bit integer
+// mantissas in the reductions (ProdAcc, ProdStateQ; no FP64 instruction per
+// element), FP64 ones in [0.5, 1) in finished states (ProdState) and in
+// reduce_by_index over FP64 values.
 #pragma once
 
 #include <stdint.h>
@@ -30,8 +30,7 @@ __device__ __forceinline__ void split_pow2(double x, double& m, int64_t& e) {
     e = (int64_t)(ex - 1022 + adj);
 }
 
-// FP32 x != 0 finite:  x = m * 2^e, 0.5 <= |m| < 1, with m as an FP32 and
-// as an FP64 (formed from the bits: no conversion instruction)
+// FP32 x != 0 finite:  x = m * 2^e, 0.5 <= |m| < 1
 __device__ __forceinline__ void split_pow2_f32m(float x, float& m, int& e) {
     int bits = __float_as_int(x);
     int ex = (bits >> 23) & 0xff;
@@ -44,15 +43,6 @@ __device__ __forceinline__ void split_pow2_f32m(float x, float& m, int& e) {
     }
     m = __int_as_float((bits & ~(0xff << 23)) | (126 << 23));
     e = ex - 126 + adj;
-}
-__device__ __forceinline__ void split_pow2_f32(float x, double& m, int64_t& e) {
-    float mf;
-    int ef;
-    split_pow2_f32m(x, mf, ef);
-    const int b = __float_as_int(mf);
-    const unsigned long long sign = (unsigned long long)((unsigned)b & 0x80000000u) << 32;
-    m = __longlong_as_double((long long)(sign | (1022ULL << 52) | ((unsigned long long)(b & 0x7fffff) << 29)));
-    e = ef;
 }
 
 // Renormalise m (nonzero, normal) into [0.5, 1), moving its exponent into e.
