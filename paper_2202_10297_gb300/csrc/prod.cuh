@@ -65,9 +65,11 @@ struct ProdState {
 
 // (zero count, lowest zero index, product of the nonzeros) of a range, as the
 // reductions combine it: the product is M * 2^(E - 63) with M in [2^63, 2^64),
-// its sign a parity.  A product keeps its top 64 bits with the last one set
-// (below), so a factor adds a relative error below 2^-62 of either sign, and
-// 2^26 factors stay within 1e-14 (truncation alone drifts one way: 5e-12).
+// its sign a parity.  A factor's product keeps its top 64 bits with the last one
+// set (below), so a factor adds a relative error below 2^-62 of either sign, and
+// 2^26 factors stay within 1e-14 (truncation alone drifts one way: 5e-12).  Two
+// states combine by rounding to nearest: a tree of exact products stays exact,
+// the neutral states of idle threads among them.
 struct ProdStateQ {
     unsigned long long M;
     long long E;
@@ -174,8 +176,13 @@ struct ProdAcc {
 
 __device__ __forceinline__ ProdStateQ ProdStateQ::comb(const ProdStateQ& x, const ProdStateQ& y) {
     ProdStateQ r;
-    int de;
-    r.M = top_mul(x.M, y.M, de);
+    const unsigned long long hi = __umul64hi(x.M, y.M), lo = x.M * y.M;  // hi in [2^62, 2^64 - 2]
+    int de = (int)(hi >> 63);
+    r.M = de ? hi + (lo >> 63) : ((hi << 1) | (lo >> 63)) + ((lo >> 62) & 1ull);
+    if (r.M == 0ull) {  // rounded up to the next power of two
+        r.M = 1ull << 63;
+        de = 1;
+    }
     r.E = x.E + y.E + de;
     r.nz = x.nz + y.nz;
     r.first = x.first < y.first ? x.first : y.first;
