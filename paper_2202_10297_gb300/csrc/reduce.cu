@@ -351,28 +351,29 @@ __device__ __forceinline__ void prod_adjoint_body(const ReduceArgs& A, const Pro
         if (i < A.n) abar[i] = A.accumulate ? abar[i] + one(a[i]) : one(a[i]);
         return;
     }
-    // zeros among the elements (or ybar = 0): 0, and the only zero's own adjoint
+    // zeros among the elements (or ybar = 0): 0, and the only zero's own adjoint,
+    // which joins the accumulated value before it is rounded to T
     const int64_t at = st.nz == 1 && yb != 0.0 ? st.first : -1;
-    auto value = [&](int64_t i) -> T { return i == at ? (T)ldexp_clamped(kq, st.e + ye) : T(0); };
+    auto put = [&](int64_t i) -> T {
+        const double c = i == at ? ldexp_clamped(kq, st.e + ye) : 0.0;
+        return (T)(A.accumulate ? (double)abar[i] + c : c);
+    };
     constexpr int V = Vec16<T>::N;
     const int64_t nv = A.n / V;
     for (int64_t v = t0; v < nv; v += stride) {
+        T* p = abar + v * V;
         Vec16<T> o;
-#pragma unroll
-        for (int k = 0; k < V; ++k) o.v[k] = T(0);
         if (at / V == v && at >= 0) {
 #pragma unroll
-            for (int k = 0; k < V; ++k) o.v[k] = value(v * V + k);
-        }
-        T* p = abar + v * V;
-        if (A.accumulate) {
+            for (int k = 0; k < V; ++k) o.v[k] = put(v * V + k);
+        } else {
 #pragma unroll
-            for (int k = 0; k < V; ++k) o.v[k] += p[k];
+            for (int k = 0; k < V; ++k) o.v[k] = A.accumulate ? p[k] : T(0);
         }
         st_vec(p, o);
     }
     const int64_t i = nv * V + t0;
-    if (i < A.n) abar[i] = A.accumulate ? abar[i] + value(i) : value(i);
+    if (i < A.n) abar[i] = put(i);
 }
 
 template <class T>

@@ -42,3 +42,23 @@ def test_batch_of_exact_products(n):
     B.run()
     r = B.aux_records()[0]
     assert (r["mant"], r["exp2"], r["sign"]) == (-0.75, 1, -1)
+
+
+# the only zero's adjoint 1 + 2^-14 + 2^-30 is not an FP32 value: it is added to
+# the accumulated -(1 + 2^-14) before the sum is rounded
+@pytest.mark.parametrize("n", [3, 4, 7, 4096, 300001])
+@pytest.mark.parametrize("at", [0, -1])
+def test_zero_adjoint_joins_the_accumulated_value(n, at):
+    from paper_2202_10297_gb300 import adpar as A
+    a = np.ones(n, np.float32)
+    a[1] = 1 + 2.0 ** -15
+    a[at] = 0
+    rest = 1 + 2.0 ** -15
+    init = torch.full((n,), 3.0, device="cuda")
+    init[at] = -(1 + 2.0 ** -14)
+    ybar = torch.tensor([1 + 2.0 ** -15], device="cuda")
+    out = A.adpar_vjp_reduce("mul", torch.from_numpy(a).cuda(), ybar, abar=init, accumulate=True)["abar"].cpu()
+    assert out[at].item() == rest * rest - (1 + 2.0 ** -14) == 2.0 ** -30
+    keep = torch.ones(n, dtype=torch.bool)
+    keep[at] = False
+    assert torch.all(out[keep] == 3.0)
