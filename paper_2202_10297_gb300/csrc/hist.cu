@@ -81,7 +81,7 @@ struct HistArgs {
     long long* pf;            // [m] * : lowest zero index
     // * over FP32 values by logarithm sums (hist_logprod.cuh): pz, pf and
     ulonglong2* acc;  // [m] the bins' words
-    ulonglong2* tab;  // [kLogTab]
+    long long* whole; // [m] their integer parts (arrays of several chunks)
     BinQ* binq;       // [m] factors of the adjoint
     // * : per-block partial states of the shared-memory bins [0, hw), merged
     // by hist_prod_merge_kernel ([blocks][hw] each)
@@ -351,8 +351,7 @@ __device__ __forceinline__ void read_bin(const HistArgs& A, int64_t b, double& m
     e = A.pe[b] + ee;
 }
 
-// Bin tiers of the * recompute over FP64 values (and FP32 arrays of 2^32
-// elements and more):
+// Bin tiers of the * recompute over FP64 values:
 //   [0, H)       warp-private copies: lanes of a warp that hit the same bin
 //                are serialised into rounds (__match_any_sync picks one
 //                leader per bin per round), so every update is a plain
@@ -373,7 +372,7 @@ struct alignas(16) WBin {
     unsigned Z;
 };
 
-template <class T, class I>
+template <class I>
 __global__ void __launch_bounds__(kProdBlock, 4) hist_prod_kernel(HistArgs A) {
     extern __shared__ unsigned char smem_raw[];
     constexpr int NW = kProdBlock / 32;
@@ -400,7 +399,7 @@ __global__ void __launch_bounds__(kProdBlock, 4) hist_prod_kernel(HistArgs A) {
     WBin* myb = wb + warp * H;
     long long* myf = wf + warp * H;
     const I* inds = static_cast<const I*>(A.inds);
-    const T* vals = static_cast<const T*>(A.vals);
+    const double* vals = static_cast<const double*>(A.vals);
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     const int64_t nround = (A.n + stride - 1) / stride;  // same trip count in every lane
     for (int64_t it = 0; it < nround; ++it) {
@@ -409,7 +408,7 @@ __global__ void __launch_bounds__(kProdBlock, 4) hist_prod_kernel(HistArgs A) {
         double v = 0.0;
         if (i < A.n) {
             b = ld_index(inds, i);
-            v = (double)__ldcs(vals + i);
+            v = __ldcs(vals + i);
         }
         const bool zero = v == 0.0;
         double mi = 0.5;
@@ -600,26 +599,21 @@ __global__ void __launch_bounds__(kHistBlock) hist_prod_vjp_kernel(HistArgs A) {
 }
 
 // ------------------------------------------------------------ host side
-// FP32 * by logarithm sums: within the words' range (every realistic call)
-bool use_logprod(int op, int dtype, int64_t n, int64_t m) {
-    return op == ADPAR_OP_MUL && dtype == ADPAR_F32 && n < (int64_t(1) << 32) && m < (int64_t(1) << 31);
-}
-
 struct HistLayout {
-    size_t off_key, off_idx, off_pm, off_pe, off_pz, off_pf, off_acc, off_tab, off_binq, off_part_m, off_part_e,
+    size_t off_key, off_idx, off_pm, off_pe, off_pz, off_pf, off_acc, off_whole, off_binq, off_part_m, off_part_e,
         off_part_f, off_part_z, total;
 };
 
-HistLayout hist_layout(int op, int dtype, int64_t n, int64_t m) {
+HistLayout hist_layout(int op, int dtype, int64_t m) {
     HistLayout L{};
     size_t o = sizeof(WsHeader);
     const size_t mm = (size_t)std::max<int64_t>(m, 1);
     if (op == ADPAR_OP_MIN || op == ADPAR_OP_MAX) {
         L.off_key = o; o = round_up(o + mm * 8, 256);
         if (dtype == ADPAR_F64) { L.off_idx = o; o = round_up(o + mm * 8, 256); }
-    } else if (use_logprod(op, dtype, n, m)) {
-        L.off_tab = o; o = round_up(o + kLogTab * 16, 256);
+    } else if (op == ADPAR_OP_MUL && dtype == ADPAR_F32) {
         L.off_acc = o; o = round_up(o + mm * 16, 256);
+        L.off_whole = o; o = round_up(o + mm * 8, 256);
         L.off_pf = o; o = round_up(o + mm * 8, 256);
         L.off_pz = o; o = round_up(o + mm * 4, 256);
         L.off_binq = o; o = round_up(o + mm * sizeof(BinQ), 256);
@@ -691,45 +685,47 @@ int run_hist(HistArgs A, cudaStream_t s) {
     }
     case ADPAR_OP_MUL: {
         if constexpr (sizeof(T) == 4) {
-            if (A.acc) {
-                LogProdArgs G{A.n, A.m, static_cast<const float*>(A.vals), A.inds, A.acc, A.pz,
-                              A.bin_aux ? A.pf : nullptr, A.tab};
-                const int gi = (int)std::max<int64_t>(
-                    8, std::min<int64_t>((A.m + 255) / 256, (int64_t)sms * 8));
-                hist_logprod_init_kernel<<<gi, 256, 0, s>>>(A.hdr, G, A.tab);
-                const int hot = (int)std::min<int64_t>(A.m, kLogHot);
-                const int H = (int)std::min<int64_t>(A.m, kLogHot + kLogSlots);
-                const size_t sh = kLogTab * 16 + (size_t)(31 * hot + H) * 16;
-                const int gp = (int)std::max<int64_t>(
-                    1, std::min<int64_t>((A.n + 4 * kLogThreads - 1) / (4 * kLogThreads), sms));
-                hist_logprod_kernel<I><<<gp, kLogThreads, sh, s>>>(G);
-                const bool map = !A.primal_only && !A.logdomain && A.n > 0;
-                hist_logprod_bins_kernel<<<gridM, 256, 0, s>>>(G, static_cast<const float*>(A.hsbar),
-                                                               map ? A.binq : nullptr,
-                                                               static_cast<float*>(A.hs_out), A.bin_aux,
-                                                               A.logdomain);
-                if (map) {
-                    const int g = (int)std::max<int64_t>(
-                        1, std::min<int64_t>((A.n / 4 + 255) / 256, (int64_t)sms * 8));
-                    hist_logprod_vjp_kernel<I><<<g, 256, 0, s>>>(G, A.binq, static_cast<float*>(A.valsbar),
-                                                                 A.accumulate);
-                } else if (!A.primal_only) {
-                    hist_prod_vjp_kernel<T, I><<<gridN, kHistBlock, 0, s>>>(A);
-                }
-                break;
+            const int64_t chunk = std::min<int64_t>(kLogChunk, (int64_t)sms << 22);  // a multiple of 4
+            const bool chunks = A.n > chunk;
+            LogProdArgs G{A.n, A.m, static_cast<const float*>(A.vals), A.inds, A.acc, chunks ? A.whole : nullptr,
+                          A.pz, A.bin_aux ? A.pf : nullptr};
+            hist_logprod_init_kernel<<<gridM, 256, 0, s>>>(A.hdr, G);
+            const int hot = (int)std::min<int64_t>(A.m, kLogHot);
+            const int H = (int)std::min<int64_t>(A.m, kLogHot + kLogSlots);
+            const size_t sh = kLogTab * 16 + (size_t)(31 * hot + H) * 16;
+            // bins of 2^31 and more exist only where an index can name one
+            auto kernel = hist_logprod_kernel<I, int>;
+            if (sizeof(I) == 8 && A.m > INT32_MAX) kernel = hist_logprod_kernel<I, I>;
+            for (int64_t lo = 0; lo < A.n; lo += chunk) {
+                const int64_t len = std::min<int64_t>(chunk, A.n - lo);
+                const int gp = (int)std::min<int64_t>((len + 4 * kLogThreads - 1) / (4 * kLogThreads), sms);
+                if (lo > 0) hist_logprod_carry_kernel<<<gridM, 256, 0, s>>>(G);
+                kernel<<<gp, kLogThreads, sh, s>>>(G, lo, lo + len);
             }
+            const bool map = !A.primal_only && !A.logdomain && A.n > 0;
+            hist_logprod_bins_kernel<<<gridM, 256, 0, s>>>(G, static_cast<const float*>(A.hsbar),
+                                                           map ? A.binq : nullptr, static_cast<float*>(A.hs_out),
+                                                           A.bin_aux, A.logdomain);
+            if (map) {
+                const int g = (int)std::max<int64_t>(
+                    1, std::min<int64_t>((A.n / 4 + 255) / 256, (int64_t)sms * 8));
+                hist_logprod_vjp_kernel<I><<<g, 256, 0, s>>>(G, A.binq, static_cast<float*>(A.valsbar),
+                                                             A.accumulate);
+            } else if (!A.primal_only) {
+                hist_prod_vjp_kernel<T, I><<<gridN, kHistBlock, 0, s>>>(A);
+            }
+        } else {
+            const int64_t h1 = std::min<int64_t>(A.m, kProdWarpBins);
+            const int64_t h2 = std::max<int64_t>(0, std::min<int64_t>(A.m - h1, kProdBlockBins));
+            const size_t sh = (size_t)h1 * 24 * (kProdBlock / 32) + (size_t)h2 * 28;
+            const int gridP = (int)std::max<int64_t>(
+                1, std::min<int64_t>((A.n + kProdBlock - 1) / kProdBlock, std::min<int64_t>(sms * 4, kProdMaxGrid)));
+            A.hw = h1 + h2;
+            hist_prod_kernel<I><<<gridP, kProdBlock, sh, s>>>(A);
+            if (A.hw > 0) hist_prod_merge_kernel<<<(unsigned)((A.hw * 32 + 255) / 256), 256, 0, s>>>(A, gridP);
+            if (A.hs_out || A.bin_aux) hist_prod_bins_kernel<T><<<gridM, 256, 0, s>>>(A);
+            if (!A.primal_only) hist_prod_vjp_kernel<T, I><<<gridN, kHistBlock, 0, s>>>(A);
         }
-        const int64_t h1 = std::min<int64_t>(A.m, kProdWarpBins);
-        const int64_t h2 = std::max<int64_t>(0, std::min<int64_t>(A.m - h1, kProdBlockBins));
-        const size_t sh = (size_t)h1 * 24 * (kProdBlock / 32) + (size_t)h2 * 28;
-        const int gridP = (int)std::max<int64_t>(
-            1, std::min<int64_t>((A.n + kProdBlock - 1) / kProdBlock, std::min<int64_t>(sms * 4, kProdMaxGrid)));
-        A.hw = h1 + h2;
-        hist_prod_kernel<T, I><<<gridP, kProdBlock, sh, s>>>(A);
-        if (A.hw > 0) hist_prod_merge_kernel<<<(unsigned)((A.hw * 32 + 255) / 256), 256, 0, s>>>(A, gridP);
-        if (A.hs_out || A.bin_aux) hist_prod_bins_kernel<T><<<gridM, 256, 0, s>>>(A);
-        if (A.primal_only) break;
-        hist_prod_vjp_kernel<T, I><<<gridN, kHistBlock, 0, s>>>(A);
         break;
     }
     default:
@@ -745,9 +741,12 @@ template <class T, class I>
 void configure_smem() {
     // the recompute kernels use up to 64 KB of dynamic shared memory
     cudaFuncSetAttribute(hist_add_primal_kernel<T, I>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024);
-    cudaFuncSetAttribute(hist_prod_kernel<T, I>, cudaFuncAttributeMaxDynamicSharedMemorySize, 112 * 1024);
-    if constexpr (sizeof(T) == 4) {
-        cudaFuncSetAttribute(hist_logprod_kernel<I>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLogSmem);
+    if constexpr (sizeof(T) == 8) {
+        cudaFuncSetAttribute(hist_prod_kernel<I>, cudaFuncAttributeMaxDynamicSharedMemorySize, 112 * 1024);
+    } else {
+        cudaFuncSetAttribute(hist_logprod_kernel<I, int>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLogSmem);
+        if constexpr (sizeof(I) == 8)
+            cudaFuncSetAttribute(hist_logprod_kernel<I, I>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLogSmem);
         for (auto f : {hist_arg_f32_kernel<I, true, true>, hist_arg_f32_kernel<I, true, false>,
                        hist_arg_f32_kernel<I, false, true>, hist_arg_f32_kernel<I, false, false>})
             cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024);
@@ -756,11 +755,11 @@ void configure_smem() {
 
 }  // namespace
 
-size_t hist_workspace_size(adpar_opdesc d, int64_t n, int64_t m) {
+size_t hist_workspace_size(adpar_opdesc d, int64_t m) {
     if (m < 0 || (d.dtype != ADPAR_F32 && d.dtype != ADPAR_F64)) return (size_t)-1;
     if (d.op != ADPAR_OP_ADD && d.op != ADPAR_OP_MUL && d.op != ADPAR_OP_MIN && d.op != ADPAR_OP_MAX)
         return (size_t)-1;
-    return hist_layout(d.op, d.dtype, n, m).total;
+    return hist_layout(d.op, d.dtype, m).total;
 }
 
 }  // namespace adpar
@@ -789,7 +788,7 @@ int hist_impl(adpar_opdesc d, int64_t n, int64_t m, const void* vals, const void
     const void* ptrs[] = {vals, inds, hsbar, valsbar, hs_out};
     for (const void* p : ptrs)
         if (p && !aligned16(p)) return ADPAR_ERR_ALIGN;
-    const HistLayout L = hist_layout(d.op, d.dtype, n, m);
+    const HistLayout L = hist_layout(d.op, d.dtype, m);
     if (!work || work_bytes < L.total || (reinterpret_cast<uintptr_t>(work) & 255u)) return ADPAR_ERR_WORKSPACE;
     if (n == 0 && m == 0) return ADPAR_OK;
     HistArgs A{};
@@ -820,7 +819,7 @@ int hist_impl(adpar_opdesc d, int64_t n, int64_t m, const void* vals, const void
     }
     if (L.off_acc) {
         A.acc = reinterpret_cast<ulonglong2*>(w + L.off_acc);
-        A.tab = reinterpret_cast<ulonglong2*>(w + L.off_tab);
+        A.whole = reinterpret_cast<long long*>(w + L.off_whole);
     }
     if (L.off_pm) {
         A.pm = reinterpret_cast<double*>(w + L.off_pm);

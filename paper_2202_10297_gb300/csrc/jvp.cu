@@ -29,7 +29,7 @@
 
 namespace adpar {
 size_t reduce_workspace_size(adpar_opdesc d);
-size_t hist_workspace_size(adpar_opdesc d, int64_t n, int64_t m);
+size_t hist_workspace_size(adpar_opdesc d, int64_t m);
 size_t kmeans_workspace_size(int64_t k);
 
 namespace {
@@ -288,9 +288,9 @@ JvpReduceLayout jvp_reduce_layout(adpar_opdesc d) {
 struct JvpHistLayout {
     size_t hist, off_hs, off_arg, off_aux, off_S, total;
 };
-JvpHistLayout jvp_hist_layout(adpar_opdesc d, int64_t n, int64_t m) {
+JvpHistLayout jvp_hist_layout(adpar_opdesc d, int64_t m) {
     JvpHistLayout L;
-    L.hist = hist_workspace_size(d, n, m);
+    L.hist = hist_workspace_size(d, m);
     const size_t mm = (size_t)std::max<int64_t>(m, 1);
     L.off_hs = round_up(L.hist, 256);
     L.off_arg = round_up(L.off_hs + mm * 8, 256);
@@ -308,9 +308,9 @@ size_t jvp_reduce_workspace_size(adpar_opdesc d) {
     return jvp_reduce_layout(d).total;
 }
 
-size_t jvp_hist_workspace_size(adpar_opdesc d, int64_t n, int64_t m) {
-    if (m < 0 || hist_workspace_size(d, n, m) == (size_t)-1) return (size_t)-1;
-    return jvp_hist_layout(d, n, m).total;
+size_t jvp_hist_workspace_size(adpar_opdesc d, int64_t m) {
+    if (m < 0 || hist_workspace_size(d, m) == (size_t)-1) return (size_t)-1;
+    return jvp_hist_layout(d, m).total;
 }
 
 size_t kmeans_fwd_rev_workspace_size(int64_t N, int64_t k) {
@@ -385,7 +385,7 @@ extern "C" int adpar_jvp_hist(adpar_opdesc d, int64_t n, int64_t m, const void* 
     if (hsdot_aux && d.op != ADPAR_OP_MUL) return ADPAR_ERR_UNSUPPORTED;
     if ((vals && !aligned16(vals)) || (vdot && !aligned16(vdot)) || (inds && !aligned16(inds)))
         return ADPAR_ERR_ALIGN;
-    const JvpHistLayout L = jvp_hist_layout(d, n, m);
+    const JvpHistLayout L = jvp_hist_layout(d, m);
     if (!work || work_bytes < L.total || (reinterpret_cast<uintptr_t>(work) & 255u)) return ADPAR_ERR_WORKSPACE;
     if (m == 0) return ADPAR_OK;
     char* w = static_cast<char*>(work);
