@@ -21,6 +21,7 @@
 // to a third word.
 #pragma once
 
+#include <math_constants.h>
 #include <stdint.h>
 
 #include "common.cuh"
@@ -354,6 +355,18 @@ __device__ __forceinline__ float top_to_f32(unsigned long long M) {
     return __int_as_float(0x3f000000 + (int)(r - 0x800000u));
 }
 
+// M * 2^(E - 63) rounded once to FP32, to nearest even (subnormals and infinity too)
+__device__ __forceinline__ float prod_to_f32(unsigned long long M, long long E) {
+    if (E > 127) return CUDART_INF_F;
+    const bool normal = E >= -126;
+    const long long drop = normal ? 40 : 40 - 126 - E;  // bits of M below the last place
+    if (drop > 64) return 0.f;
+    unsigned r = drop == 64 ? 0u : (unsigned)(M >> drop);
+    const unsigned long long rest = M << (64 - drop);
+    r += rest > (1ull << 63) || (rest == (1ull << 63) && (r & 1u)) ? 1u : 0u;
+    return __uint_as_float((normal ? (unsigned)(E + 126) << 23 : 0u) + r);
+}
+
 // per bin: the recomputed product and what the call asked for
 __global__ void hist_logprod_bins_kernel(LogProdArgs A, const float* hsbar, BinQ* binq, float* hs_out,
                                          adpar_prod_aux* aux, int keep_pow2) {
@@ -365,7 +378,7 @@ __global__ void hist_logprod_bins_kernel(LogProdArgs A, const float* hsbar, BinQ
         logprod_decode(A.acc[b], A.whole ? A.whole[b] : 0, M, E, sign);
         const unsigned nz = A.pz[b];
         if (hs_out) {
-            const float p = scale_pow2f(top_to_f32(M), E + 1);
+            const float p = prod_to_f32(M, E);
             hs_out[b] = nz ? 0.f : (sign ? -p : p);
         }
         if (binq) {
