@@ -31,6 +31,7 @@ constexpr bool kVecPrimal = Op::kNeedPrimal || Op::kCoefNeedsPrimal || !Op::kCoe
 
 struct VecArgs {
     int64_t n, d, C;  // rows, columns, chunks
+    int flat;         // threads run over (chunk, column) pairs, not blocks over columns
     const void* a;
     const void* b;
     const void* ya;
@@ -42,9 +43,29 @@ struct VecArgs {
     void* aggL;  // [C][d] L: chunk aggregates, then exclusive suffixes
 };
 
+// This thread's chunk and column.  Blocks lie along the columns, a grid row per
+// chunk; with few columns (flat) consecutive threads take consecutive (chunk,
+// column) pairs, so that narrow arrays do not leave most lanes idle.
+// FLATFIGS
+constexpr int64_t kVecFlat = 1024;
+template <int B>
+__device__ __forceinline__ bool vec_place(const VecArgs& V, int64_t& c, int64_t& col) {
+    if (V.flat) {
+        const int64_t i = blockIdx.x * (int64_t)B + threadIdx.x;
+        if (V.C * V.d <= UINT32_MAX) c = (unsigned)i / (unsigned)V.d;
+        else c = i / V.d;
+        col = i - c * V.d;
+        return c < V.C;
+    }
+    c = blockIdx.y;
+    col = blockIdx.x * (int64_t)B + threadIdx.x;
+    return col < V.d;
+}
+
 // rows whose loads a thread has in flight at once
-constexpr int kVecU = 8;     // output pass
-constexpr int kVecUAgg = 4;  // aggregates
+constexpr int kVecU = 8;  // output pass
+template <class Op>
+constexpr int kVecUAgg = Op::kWidth == 2 || Op::kCoefOne ? 4 : 8;  // aggregates (LINREC loads two or three arrays)
 
 // p[i], p[i + d], .. for U rows from `row` on (pad past the last row)
 template <int U, class T>
@@ -59,9 +80,9 @@ __device__ __forceinline__ void vec_rows(const void* p, const VecArgs& V, int64_
 template <class Op, class T>
 __global__ void __launch_bounds__(kVecBlock, 6) vec_primal_agg_kernel(VecArgs V) {
     using P = typename Op::P;
-    constexpr int W = Op::kWidth, U = kVecUAgg;
-    const int64_t col = blockIdx.x * (int64_t)kVecBlock + threadIdx.x, c = blockIdx.y;
-    if (col >= V.d) return;
+    constexpr int W = Op::kWidth, U = kVecUAgg<Op>;
+    int64_t c, col;
+    if (!vec_place<kVecBlock>(V, c, col)) return;
     const int64_t r0 = c * kVecR;
     P acc = Op::pid();
 #pragma unroll 1
@@ -78,11 +99,16 @@ __global__ void __launch_bounds__(kVecBlock, 6) vec_primal_agg_kernel(VecArgs V)
 // Turns the chunk aggregates of 32 columns into exclusive prefixes (REV:
 // exclusive suffixes, composed right to left).  Thread (x, y) of a 32 x G block
 // folds group y of column x's chunks (neighbouring lanes read neighbouring
-// columns), the groups' folds are scanned by shuffles, a warp per column, and
-// each thread runs through its chunks again.  8 chunks are loaded at a time; G
-// is a group per 8 chunks, up to 32.
+// columns), the groups' folds are scanned, and each thread runs through its
+// chunks again.  8 chunks are loaded at a time; G is a group per 8 chunks, up to
+// 32.  The groups' folds: by shuffles, a warp per column, where there are many in
+// FP32; few of them, and FP64 ones (a warp's combination takes the FP64 pipe of
+// the SM 32 cycles, and 32 columns take five steps each), one after another by a
+// thread per column.  FP64 max over 500 x 64, by shuffles and now: the call 57 and
+// 39 us; over 500 x 2048, 64 and 49 us (4 or 2 chunks a group: no faster).
 constexpr int kVecG = 32;
-template <class S, bool REV, class Comb>
+constexpr int kVecSerialG = 8;
+template <bool F64, class S, bool REV, class Comb>
 __device__ __forceinline__ void vec_scan_columns(S* agg, int64_t C, int64_t d, S* s_tot, const S& ident, Comb comb) {
     const int x = threadIdx.x & 31, y = threadIdx.x >> 5, G = blockDim.x >> 5;
     const int64_t col = blockIdx.x * (int64_t)32 + x;
@@ -98,12 +124,24 @@ __device__ __forceinline__ void vec_scan_columns(S* agg, int64_t C, int64_t d, S
 #pragma unroll
                 for (int u = 0; u < 8; ++u) v[u] = q + u < hi ? *at(q + u) : ident;
 #pragma unroll
-                for (int u = 0; u < 8; ++u) run = comb(run, v[u]);
+                for (int u = 0; u < 8; ++u) {
+                    if (q + u >= hi) break;
+                    run = comb(run, v[u]);
+                }
             }
         }
         s_tot[y * 33 + x] = run;
         __syncthreads();
-        for (int w = y; w < 32; w += G) {  // lane x holds group x of column w
+        const bool serial = F64 || G <= kVecSerialG;
+        if (serial && y == 0) {
+            S pre = ident;
+            for (int w = 0; w < G; ++w) {
+                const S t = s_tot[w * 33 + x];
+                s_tot[w * 33 + x] = pre;
+                pre = comb(pre, t);
+            }
+        }
+        for (int w = serial ? 32 : y; w < 32; w += G) {  // lane x holds group x of column w
             S inc = x < G ? s_tot[x * 33 + w] : ident;
 #pragma unroll
             for (int off = 1; off < 32; off <<= 1) {
@@ -141,11 +179,11 @@ __global__ void __launch_bounds__(32 * kVecG) vec_scan_kernel(VecArgs V, int fir
     using L = Lin<T, Op::kWidth, !Op::kCoefOne>;
     extern __shared__ __align__(16) unsigned char s_dyn[];
     if (blockIdx.y + first == 0) {
-        vec_scan_columns<P, false>(static_cast<P*>(V.aggP), V.C, V.d, reinterpret_cast<P*>(s_dyn), Op::pid(),
+        vec_scan_columns<sizeof(T) == 8, P, false>(static_cast<P*>(V.aggP), V.C, V.d, reinterpret_cast<P*>(s_dyn), Op::pid(),
                                    [](const P& l, const P& r) { return Op::pcomb(l, r); });
     } else {
         // scan order is right to left: e holds later rows, l earlier ones
-        vec_scan_columns<L, true>(static_cast<L*>(V.aggL), V.C, V.d, reinterpret_cast<L*>(s_dyn), L::id(),
+        vec_scan_columns<sizeof(T) == 8, L, true>(static_cast<L*>(V.aggL), V.C, V.d, reinterpret_cast<L*>(s_dyn), L::id(),
                                   [](const L& e, const L& l) { return L::comb(e, l); });
     }
 }
@@ -192,12 +230,12 @@ __device__ __forceinline__ void vec_coefs(const VecArgs& V, int64_t row, int64_t
 // growing map of a sweep from the top, fused with the operator's, read each
 // array once and took 52 us for 23 + 40, but its FP32 results were further off)
 template <class Op, class T>
-__global__ void __launch_bounds__(kVecBlock, 6) vec_adjoint_agg_kernel(VecArgs V) {
+__global__ void __launch_bounds__(kVecBlock, Op::kCoefOne && sizeof(T) == 4 ? 8 : 6) vec_adjoint_agg_kernel(VecArgs V) {
     using P = typename Op::P;
-    constexpr int W = Op::kWidth, U = kVecUAgg;
+    constexpr int W = Op::kWidth, U = kVecUAgg<Op>;
     using L = Lin<T, W, !Op::kCoefOne>;
-    const int64_t col = blockIdx.x * (int64_t)kVecBlock + threadIdx.x, c = blockIdx.y;
-    if (col >= V.d) return;
+    int64_t c, col;
+    if (!vec_place<kVecBlock>(V, c, col)) return;
     const int64_t r0 = c * kVecR;
     uint32_t bits = 0u;
     if constexpr (Op::kCoefNeedsPrimal)
@@ -240,8 +278,9 @@ __global__ void __launch_bounds__(kVecOutBlock, 9) vec_output_kernel(VecArgs V) 
     constexpr bool kP = kVecPrimal<Op>;
     using L = Lin<T, W, !Op::kCoefOne>;
     __shared__ T s_r[kVecR * W * kVecOutBlock];  // rs_bar of the thread's rows, [row][component][thread]
-    const int64_t col = blockIdx.x * (int64_t)kVecOutBlock + threadIdx.x, c = V.C - 1 - (int64_t)blockIdx.y;
-    if (col >= V.d) return;
+    int64_t c, col;
+    if (!vec_place<kVecOutBlock>(V, c, col)) return;
+    c = V.C - 1 - c;
     const int64_t r0 = c * kVecR;
     const P carry = kP ? static_cast<const P*>(V.aggP)[c * V.d + col] : Op::pid();
     const L suf = static_cast<const L*>(V.aggL)[c * V.d + col];
@@ -322,10 +361,18 @@ int run_vec(int64_t n, int64_t d, const void* a, const void* b, const void* ya, 
     cudaMemsetAsync(w, 0, sizeof(WsHeader), s);  // the status word starts at ok
     V.aggP = w + sizeof(WsHeader);
     V.aggL = w + sizeof(WsHeader) + round_up((size_t)V.C * d * sizeof(typename Op::P), 256);
-    const dim3 g2((unsigned)((d + kVecBlock - 1) / kVecBlock), (unsigned)V.C);
-    const dim3 g5((unsigned)((d + kVecOutBlock - 1) / kVecOutBlock), (unsigned)V.C);
+    // (few blocks spread over the SMs as they are)
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    V.flat = d < kVecFlat && V.C * ((d + kVecBlock - 1) / kVecBlock) > sms;
+    auto grid = [&](int64_t block) {
+        if (V.flat) return dim3((unsigned)((V.C * d + block - 1) / block));
+        return dim3((unsigned)((d + block - 1) / block), (unsigned)V.C);
+    };
+    const dim3 g2 = grid(kVecBlock), g5 = grid(kVecOutBlock);
     const unsigned gw = (unsigned)((d + 31) / 32);  // 32 columns per block
-    const int G = (int)std::max<int64_t>(1, std::min<int64_t>(V.C / 8, kVecG));
+    const int G = (int)std::max<int64_t>(1, V.C <= 8 ? 1 : std::min<int64_t>(V.C / 8 + 1, kVecG));
     const size_t sh = std::max(sizeof(typename Op::P), sizeof(L)) * 33 * G;
     constexpr bool kTwo = kVecPrimal<Op> && !Op::kCoefNeedsPrimal;  // both scans from one launch
     if constexpr (kVecPrimal<Op>) vec_primal_agg_kernel<Op, T><<<g2, kVecBlock, 0, s>>>(V);
