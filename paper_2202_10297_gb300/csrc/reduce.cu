@@ -506,7 +506,9 @@ int run_reduce(ReduceArgs A, int op, cudaStream_t s) {
         const int gp = (int)std::max<int64_t>(1, std::min<int64_t>((A.n + per - 1) / per, kProdGrid));
         reduce_prod_kernel<T><<<gp, kRedBlock, 0, s>>>(A);
         if (A.primal_only) break;
-        prod_adjoint_kernel<T><<<gp, kRedBlock, 0, s>>>(A);
+        // the log domain's threads form two FP64 logarithms of their own: four elements each
+        const int ga = A.logdomain ? (int)std::max<int64_t>(1, std::min<int64_t>((A.n + 1023) / 1024, kProdGrid)) : gp;
+        prod_adjoint_kernel<T><<<ga, kRedBlock, 0, s>>>(A);
         break;
     }
     default:
