@@ -32,11 +32,11 @@ __device__ __forceinline__ int64_t ldi(const I* p, int64_t j) {
 // last): every thread goes through its indices once per region and touches only
 // those in it, so a line is fetched and written back once for all of its
 // indices, at the price of reading the indices once per region.
-// Worth it when a 64-byte line holds an index or more on average (below, nothing
-// is shared) and for 8 regions at most (16: 6.7 ms against 5.2 ms in one, 2^26
-// indices into 1 GB); not when the indices are local already (sorted, say):
-// each block looks at 256 pairs 64 apart, the same pairs in all blocks, and
-// takes one region when most lie close.
+// Worth it when a 64-byte line holds enough indices on average, how many
+// depending on the pass (RegionRule below), and for few regions (16: 6.7 ms
+// against 5.2 ms in one, 2^26 indices into 1 GB); not when the indices are local
+// already (sorted, say): each block looks at 256 pairs 64 apart, the same pairs in
+// all blocks, and takes one region when most lie close.
 // Random accesses of 4 bytes on a GB300, in G/s, within 64 MB / over 256 MB:
 // loads 286 / 77, stores 209 / 33, exchanges 134 / 36.  Forward and VJP through
 // autograd, 2^24 indices into 2^26 FP32 (of it 170 us for the two copies of the
@@ -45,25 +45,57 @@ __device__ __forceinline__ int64_t ldi(const I* p, int64_t j) {
 constexpr int64_t kRegionBytes = int64_t(64) << 20;
 constexpr int64_t kMaxRegions = 8;
 constexpr int64_t kLocalBytes = int64_t(1) << 20;
+constexpr int64_t kDenseBytes = 64 * 24;  // 64 indices within this many bytes
+constexpr int64_t kDenseMin = int64_t(24) << 20;  // bytes of vs (fewer: exchanges within L2 are as fast)
 // blocks per SM, all resident: the grid goes through the regions together
 constexpr int kScatBlocks = 6;
 
+// When a pass goes by regions: target bytes, indices per 64-byte line, regions.
+// Time by regions over time in one, targets of 128 / 256 MB, FP32:
+//   VJP                       1 index per line 1.2 / 0.9, 2 per line 0.9 / 0.8
+//   forward                   1 per line 1.4 / 1.1, 2 per line 1.0 / 0.8
+//   forward, keeping the old  2 per line 1.0 / 1.0, 4 per line 0.8 / 0.9; of 440 MB
+//     values                  1.2 (FP64 4 per line 0.9 / 1.0, 8 per line 0.8 / 1.0)
+struct RegionRule {
+    int64_t min_bytes;
+    int per_line;
+    int64_t max_regions;
+};
+constexpr RegionRule kVjpRule{2 * kRegionBytes, 1, kMaxRegions};
+constexpr RegionRule kFwdRule{2 * kRegionBytes, 2, kMaxRegions};
+constexpr RegionRule save_rule(size_t esz) { return {kRegionBytes * 3 / 2, esz == 4 ? 4 : 8, 5}; }
+
 // elements per region (below 2^32): all of n where one region will do
-inline int64_t region_elems(int64_t n, int64_t m, size_t esz) {
+inline int64_t region_elems(int64_t n, int64_t m, size_t esz, const RegionRule& rule) {
     const int64_t bytes = n * (int64_t)esz;
     const int64_t regions = (bytes + kRegionBytes - 1) / kRegionBytes;
-    if (bytes < 2 * kRegionBytes || regions > kMaxRegions || m < 4096 || m * 64 < bytes)
+    if (bytes < rule.min_bytes || regions > rule.max_regions || m < 4096 || m * 64 < bytes * rule.per_line)
         return std::min<int64_t>(std::max<int64_t>(n, 1), int64_t(1) << 31);
     return ((n + regions - 1) / regions + 31) / 32 * 32;
 }
+// A target that just outgrows L2 (129 MB) and few indices per line: exchanges lose
+// to a load and a store per index (FP32, 96 to 224 MB, up to 1.13 times; FP64 1.17)
+inline bool beyond_l2(int64_t n, size_t esz) {
+    const int64_t bytes = n * (int64_t)esz;
+    return bytes >= kRegionBytes * 3 / 2 && bytes < kRegionBytes * 7 / 2;
+}
 
-// the region size this launch uses (the same in every block); all threads call it
+// the region size this launch uses (the same in every block); all threads call
+// it.  dense, where asked for: neighbouring indices share lines, as sorted ones
+// into a quarter of FP32 do (exchanges then take up to 1.15 times as long as a load
+// and a store, and 0.9 where only a 16th is written).
 template <class I>
-__device__ __forceinline__ int64_t pick_region(const I* is, int64_t n, int64_t m, int64_t region, int esz) {
-    if (region >= n || region == int64_t(1) << 31) return region;
+__device__ __forceinline__ int64_t pick_region(const I* is, int64_t n, int64_t m, int64_t region, int esz,
+                                               bool* dense = nullptr) {
+    const bool one = region >= n || region == int64_t(1) << 31;
+    if (dense) *dense = false;
+    if (one && !(dense && m * esz >= kDenseMin)) return region;
     const int64_t p = (int64_t)threadIdx.x * ((m - 64) / blockDim.x);
-    const int64_t d = (int64_t)is[p + 64] - (int64_t)is[p];
-    const int near = __syncthreads_count((d < 0 ? -d : d) <= kLocalBytes / esz);
+    int64_t d = (int64_t)is[p + 64] - (int64_t)is[p];
+    if (d < 0) d = -d;
+    if (dense && m * esz >= kDenseMin) *dense = 2 * __syncthreads_count(d <= kDenseBytes / esz) >= (int)blockDim.x;
+    if (one) return region;
+    const int near = __syncthreads_count(d <= kLocalBytes / esz);
     return 2 * near >= (int)blockDim.x ? (n < (int64_t(1) << 31) ? n : int64_t(1) << 31) : region;
 }
 
@@ -230,13 +262,38 @@ __global__ void __launch_bounds__(kBlk) map_acc_kernel(MapAccArgs<T> A) {
     }
 }
 
+// A load and a store per index, U indices per thread and step.
+template <int U, class T, class I>
+__device__ __forceinline__ void save_plain(int64_t n, int64_t m, const I* is, const T* vs, T* ys, T* xs_saved) {
+    const int64_t stride = (int64_t)gridDim.x * (kBlk * U);
+    for (int64_t j = blockIdx.x * (int64_t)(kBlk * U) + threadIdx.x; j < m; j += stride) {
+        I k[U];
+        T o[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) k[u] = j + u * kBlk < m ? __ldcs(is + j + u * kBlk) : I(-1);
+#pragma unroll
+        for (int u = 0; u < U; ++u) o[u] = k[u] >= 0 && k[u] < n ? ys[k[u]] : T(0);
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (j + u * kBlk >= m) break;
+            xs_saved[j + u * kBlk] = o[u];
+            if (k[u] >= 0 && k[u] < n) ys[k[u]] = __ldcs(vs + j + u * kBlk);
+        }
+    }
+}
+
 // primal of scatter (Sec. 5.3's forward sweep): xs_saved[j] = ys[is_j]
 // (optional), then ys[is_j] = vs[j], in place; by regions as above
 template <class T, class I, bool SAVE>
 __global__ void __launch_bounds__(kBlk, kScatBlocks) scatter_fwd_kernel(int64_t n, int64_t m, const I* is, const T* vs,
                                                                        T* ys, T* xs_saved, int64_t region_arg) {
     constexpr int U = kScatU;
-    const int64_t region = pick_region(is, n, m, region_arg, (int)sizeof(T));
+    bool dense = false;
+    const int64_t region = pick_region(is, n, m, region_arg, (int)sizeof(T), SAVE ? &dense : nullptr);
+    if (SAVE && dense) {
+        save_plain<kScatU>(n, m, is, vs, ys, xs_saved);
+        return;
+    }
     const int64_t last = n > 0 ? (n - 1) / region * region : 0;
     for (int64_t base = last; base >= 0; base -= region) {
         const int64_t left = n - base;
@@ -259,6 +316,13 @@ __global__ void __launch_bounds__(kBlk, kScatBlocks) scatter_fwd_kernel(int64_t 
         else
             for_region<false>(is, m, n, base, size, fn, [](int64_t) {});
     }
+}
+
+// the plain loop alone (beyond_l2)
+template <class T, class I>
+__global__ void __launch_bounds__(kBlk) scatter_save_kernel(int64_t n, int64_t m, const I* is, const T* vs, T* ys,
+                                                           T* xs_saved) {
+    save_plain<1>(n, m, is, vs, ys, xs_saved);
 }
 
 // primal of map: xs[j] = g(as[is_j, :], ws[j, :]) (0 for an index out of range)
@@ -320,7 +384,7 @@ extern "C" int adpar_vjp_scatter(int dtype, int64_t n, int64_t m, const void* is
     if (m == 0) return ADPAR_OK;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((m / kScatU + kBlk) / kBlk, (int64_t)sm_count() * kScatBlocks));
-    const int64_t region = region_elems(n, m, dtype == ADPAR_F64 ? 8 : 4);
+    const int64_t region = region_elems(n, m, dtype == ADPAR_F64 ? 8 : 4, kVjpRule);
     const int acc = (flags & ADPAR_ACCUMULATE) ? 1 : 0;
     void* ys = restore ? ys_restore : nullptr;
 #define ADPAR_SCATTER_RA(T, I, R, A)                                                                             \
@@ -403,11 +467,19 @@ extern "C" int adpar_scatter(int dtype, int64_t n, int64_t m, const void* is, in
     if (m == 0) return ADPAR_OK;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((m / kScatU + kBlk) / kBlk, (int64_t)sm_count() * kScatBlocks));
-    const int64_t region = region_elems(n, m, dtype == ADPAR_F64 ? 8 : 4);
+    const size_t esz = dtype == ADPAR_F64 ? 8 : 4;
+    const int64_t region = region_elems(n, m, esz, xs_saved_out ? save_rule(esz) : kFwdRule);
+    const bool plain = xs_saved_out && region >= n && beyond_l2(n, esz);
+    const int grid1 = (int)std::max<int64_t>(1, std::min<int64_t>((m + kBlk - 1) / kBlk, (int64_t)sm_count() * 8));
 #define ADPAR_SCAT_FWD_S(T, I, S)                                                                                 \
     scatter_fwd_kernel<T, I, S><<<grid, kBlk, 0, s>>>(n, m, static_cast<const I*>(is), static_cast<const T*>(vs), \
                                                       static_cast<T*>(ys_inout), static_cast<T*>(xs_saved_out), region)
-#define ADPAR_SCAT_FWD(T, I) (xs_saved_out ? ADPAR_SCAT_FWD_S(T, I, true) : ADPAR_SCAT_FWD_S(T, I, false))
+#define ADPAR_SCAT_SAVE(T, I)                                                                                     \
+    scatter_save_kernel<T, I><<<grid1, kBlk, 0, s>>>(n, m, static_cast<const I*>(is), static_cast<const T*>(vs),  \
+                                                     static_cast<T*>(ys_inout), static_cast<T*>(xs_saved_out))
+#define ADPAR_SCAT_FWD(T, I)                                                                             \
+    (plain ? ADPAR_SCAT_SAVE(T, I)                                                                       \
+           : (xs_saved_out ? ADPAR_SCAT_FWD_S(T, I, true) : ADPAR_SCAT_FWD_S(T, I, false)))
     if (dtype == ADPAR_F32) {
         if (itype == ADPAR_I32) ADPAR_SCAT_FWD(float, int32_t); else ADPAR_SCAT_FWD(float, int64_t);
     } else {
@@ -415,6 +487,7 @@ extern "C" int adpar_scatter(int dtype, int64_t n, int64_t m, const void* is, in
     }
 #undef ADPAR_SCAT_FWD
 #undef ADPAR_SCAT_FWD_S
+#undef ADPAR_SCAT_SAVE
     return cudaGetLastError() == cudaSuccess ? ADPAR_OK : ADPAR_ERR_CUDA;
 }
 
