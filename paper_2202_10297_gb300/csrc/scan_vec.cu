@@ -31,7 +31,6 @@ constexpr bool kVecPrimal = Op::kNeedPrimal || Op::kCoefNeedsPrimal || !Op::kCoe
 
 struct VecArgs {
     int64_t n, d, C;  // rows, columns, chunks
-    int flat;         // threads run over (chunk, column) pairs, not blocks over columns
     const void* a;
     const void* b;
     const void* ya;
@@ -43,23 +42,14 @@ struct VecArgs {
     void* aggL;  // [C][d] L: chunk aggregates, then exclusive suffixes
 };
 
-// This thread's chunk and column.  Blocks lie along the columns, a grid row per
-// chunk; with few columns (flat) consecutive threads take consecutive (chunk,
-// column) pairs, so that narrow arrays do not leave most lanes idle.
-// FLATFIGS
+// Blocks lie along the columns, a grid row per chunk; with few columns (FLAT)
+// consecutive threads take consecutive (chunk, column) pairs, so that narrow
+// arrays do not leave most lanes idle: FP64 max over 100000 x 1, 277 -> 220 us;
+// 4000 x 300, 76 -> 58 us.  Only where the blocks outnumber the SMs: 2000 x 64
+// spread over 63 SMs is faster than over 16.
 constexpr int64_t kVecFlat = 1024;
-template <int B>
-__device__ __forceinline__ bool vec_place(const VecArgs& V, int64_t& c, int64_t& col) {
-    if (V.flat) {
-        const int64_t i = blockIdx.x * (int64_t)B + threadIdx.x;
-        if (V.C * V.d <= UINT32_MAX) c = (unsigned)i / (unsigned)V.d;
-        else c = i / V.d;
-        col = i - c * V.d;
-        return c < V.C;
-    }
-    c = blockIdx.y;
-    col = blockIdx.x * (int64_t)B + threadIdx.x;
-    return col < V.d;
+__device__ __forceinline__ int64_t vec_chunk(const VecArgs& V, int64_t i) {
+    return (int64_t)((unsigned long long)i / (unsigned)V.d);  // d < kVecFlat
 }
 
 // rows whose loads a thread has in flight at once
@@ -77,12 +67,13 @@ __device__ __forceinline__ void vec_rows(const void* p, const VecArgs& V, int64_
 }
 
 // the operator's state over each chunk, top to bottom
-template <class Op, class T>
+template <class Op, class T, bool FLAT>
 __global__ void __launch_bounds__(kVecBlock, 6) vec_primal_agg_kernel(VecArgs V) {
     using P = typename Op::P;
     constexpr int W = Op::kWidth, U = kVecUAgg<Op>;
-    int64_t c, col;
-    if (!vec_place<kVecBlock>(V, c, col)) return;
+    const int64_t i = blockIdx.x * (int64_t)kVecBlock + threadIdx.x, c = FLAT ? vec_chunk(V, i) : (int64_t)blockIdx.y;
+    const int64_t col = FLAT ? i - c * V.d : i;
+    if (FLAT ? c >= V.C : col >= V.d) return;
     const int64_t r0 = c * kVecR;
     P acc = Op::pid();
 #pragma unroll 1
@@ -125,7 +116,7 @@ __device__ __forceinline__ void vec_scan_columns(S* agg, int64_t C, int64_t d, S
                 for (int u = 0; u < 8; ++u) v[u] = q + u < hi ? *at(q + u) : ident;
 #pragma unroll
                 for (int u = 0; u < 8; ++u) {
-                    if (q + u >= hi) break;
+                    if (F64 && q + u >= hi) break;
                     run = comb(run, v[u]);
                 }
             }
@@ -229,13 +220,14 @@ __device__ __forceinline__ void vec_coefs(const VecArgs& V, int64_t row, int64_t
 // top (Horner's order: a contracting recurrence damps the early roundings; the
 // growing map of a sweep from the top, fused with the operator's, read each
 // array once and took 52 us for 23 + 40, but its FP32 results were further off)
-template <class Op, class T>
+template <class Op, class T, bool FLAT>
 __global__ void __launch_bounds__(kVecBlock, Op::kCoefOne && sizeof(T) == 4 ? 8 : 6) vec_adjoint_agg_kernel(VecArgs V) {
     using P = typename Op::P;
     constexpr int W = Op::kWidth, U = kVecUAgg<Op>;
     using L = Lin<T, W, !Op::kCoefOne>;
-    int64_t c, col;
-    if (!vec_place<kVecBlock>(V, c, col)) return;
+    const int64_t i = blockIdx.x * (int64_t)kVecBlock + threadIdx.x, c = FLAT ? vec_chunk(V, i) : (int64_t)blockIdx.y;
+    const int64_t col = FLAT ? i - c * V.d : i;
+    if (FLAT ? c >= V.C : col >= V.d) return;
     const int64_t r0 = c * kVecR;
     uint32_t bits = 0u;
     if constexpr (Op::kCoefNeedsPrimal)
@@ -271,16 +263,16 @@ __global__ void __launch_bounds__(kVecBlock, Op::kCoefOne && sizeof(T) == 4 ? 8 
 // FP32 LINREC (59 us for its bytes); 64 registers, or one row at a time: 96 and
 // 128 us.  The scan of both aggregates takes 11 us (was 13 + 23 with a warp per
 // column); the call 245 -> 164 us.
-template <class Op, class T>
+template <class Op, class T, bool FLAT>
 __global__ void __launch_bounds__(kVecOutBlock, 9) vec_output_kernel(VecArgs V) {
     using P = typename Op::P;
     constexpr int W = Op::kWidth;
     constexpr bool kP = kVecPrimal<Op>;
     using L = Lin<T, W, !Op::kCoefOne>;
     __shared__ T s_r[kVecR * W * kVecOutBlock];  // rs_bar of the thread's rows, [row][component][thread]
-    int64_t c, col;
-    if (!vec_place<kVecOutBlock>(V, c, col)) return;
-    c = V.C - 1 - c;
+    const int64_t i = blockIdx.x * (int64_t)kVecOutBlock + threadIdx.x, f = FLAT ? vec_chunk(V, i) : (int64_t)blockIdx.y;
+    const int64_t col = FLAT ? i - f * V.d : i, c = V.C - 1 - f;
+    if (FLAT ? c < 0 : col >= V.d) return;
     const int64_t r0 = c * kVecR;
     const P carry = kP ? static_cast<const P*>(V.aggP)[c * V.d + col] : Op::pid();
     const L suf = static_cast<const L*>(V.aggL)[c * V.d + col];
@@ -346,6 +338,24 @@ size_t vec_workspace(int64_t n, int64_t d) {
            round_up((size_t)C * d * sizeof(L), 256);
 }
 
+template <class Op, class T, bool FLAT>
+void launch_vec(const VecArgs& V, cudaStream_t s) {
+    using L = Lin<T, Op::kWidth, !Op::kCoefOne>;
+    auto grid = [&](int64_t block) {
+        if (FLAT) return dim3((unsigned)((V.C * V.d + block - 1) / block));
+        return dim3((unsigned)((V.d + block - 1) / block), (unsigned)V.C);
+    };
+    const unsigned gw = (unsigned)((V.d + 31) / 32);  // 32 columns per block
+    const int G = (int)(V.C <= 8 ? 1 : std::min<int64_t>(V.C / 8 + 1, kVecG));
+    const size_t sh = std::max(sizeof(typename Op::P), sizeof(L)) * 33 * G;
+    constexpr bool kTwo = kVecPrimal<Op> && !Op::kCoefNeedsPrimal;  // both scans from one launch
+    if constexpr (kVecPrimal<Op>) vec_primal_agg_kernel<Op, T, FLAT><<<grid(kVecBlock), kVecBlock, 0, s>>>(V);
+    if constexpr (Op::kCoefNeedsPrimal) vec_scan_kernel<Op, T><<<dim3(gw, 1), 32 * G, sh, s>>>(V, 0);
+    vec_adjoint_agg_kernel<Op, T, FLAT><<<grid(kVecBlock), kVecBlock, 0, s>>>(V);
+    vec_scan_kernel<Op, T><<<dim3(gw, kTwo ? 2 : 1), 32 * G, sh, s>>>(V, kTwo ? 0 : 1);
+    vec_output_kernel<Op, T, FLAT><<<grid(kVecOutBlock), kVecOutBlock, 0, s>>>(V);
+}
+
 template <class Op, class T>
 int run_vec(int64_t n, int64_t d, const void* a, const void* b, const void* ya, const void* yb, void* abar,
             void* bbar, uint32_t flags, void* work, size_t work_bytes, cudaStream_t s) {
@@ -361,25 +371,12 @@ int run_vec(int64_t n, int64_t d, const void* a, const void* b, const void* ya, 
     cudaMemsetAsync(w, 0, sizeof(WsHeader), s);  // the status word starts at ok
     V.aggP = w + sizeof(WsHeader);
     V.aggL = w + sizeof(WsHeader) + round_up((size_t)V.C * d * sizeof(typename Op::P), 256);
-    // (few blocks spread over the SMs as they are)
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    V.flat = d < kVecFlat && V.C * ((d + kVecBlock - 1) / kVecBlock) > sms;
-    auto grid = [&](int64_t block) {
-        if (V.flat) return dim3((unsigned)((V.C * d + block - 1) / block));
-        return dim3((unsigned)((d + block - 1) / block), (unsigned)V.C);
-    };
-    const dim3 g2 = grid(kVecBlock), g5 = grid(kVecOutBlock);
-    const unsigned gw = (unsigned)((d + 31) / 32);  // 32 columns per block
-    const int G = (int)std::max<int64_t>(1, V.C <= 8 ? 1 : std::min<int64_t>(V.C / 8 + 1, kVecG));
-    const size_t sh = std::max(sizeof(typename Op::P), sizeof(L)) * 33 * G;
-    constexpr bool kTwo = kVecPrimal<Op> && !Op::kCoefNeedsPrimal;  // both scans from one launch
-    if constexpr (kVecPrimal<Op>) vec_primal_agg_kernel<Op, T><<<g2, kVecBlock, 0, s>>>(V);
-    if constexpr (Op::kCoefNeedsPrimal) vec_scan_kernel<Op, T><<<dim3(gw, 1), 32 * G, sh, s>>>(V, 0);
-    vec_adjoint_agg_kernel<Op, T><<<g2, kVecBlock, 0, s>>>(V);
-    vec_scan_kernel<Op, T><<<dim3(gw, kTwo ? 2 : 1), 32 * G, sh, s>>>(V, kTwo ? 0 : 1);
-    vec_output_kernel<Op, T><<<g5, kVecOutBlock, 0, s>>>(V);
+    // (few blocks spread over the SMs as they are)
+    if (d < kVecFlat && V.C * ((d + kVecBlock - 1) / kVecBlock) > sms) launch_vec<Op, T, true>(V, s);
+    else launch_vec<Op, T, false>(V, s);
     return cudaGetLastError() == cudaSuccess ? ADPAR_OK : ADPAR_ERR_CUDA;
 }
 
