@@ -32,7 +32,8 @@ namespace {
 
 constexpr int kHistBlock = 512;
 constexpr int kHistSmemKeys = 8192;  // 64 KB of 64-bit bin words per block
-constexpr int64_t kFilterPerBin = 64;  // FP32 min/max: elements per bin from which global words are read first
+constexpr int64_t kFilterPerBin = 256;  // FP32 min/max: elements per bin from which global words are read first
+constexpr int64_t kArgVector = 6 << 20;  // elements from which a thread takes four per step
 
 __device__ __forceinline__ uint32_t orderkey_f32(float f) {
     uint32_t u = __float_as_uint(f);
@@ -179,16 +180,18 @@ __global__ void fill_zero_kernel(void* p, int64_t nbytes) {
 
 // ------------------------------------------------------------ min / max
 // FP32: one recompute pass with packed words; fuses the zero fill of valsbar.
-// Four consecutive elements per thread and step.  2^26 elements into 2^22 bins:
-// 513 us with one element per thread and step, 440 us so (L2 atomics: 210 G/s
-// at best, 320 us); 2^25 into 256 bins 139 -> 90 us.
+// V consecutive elements per thread and step: 4 in long arrays (2^26 elements into
+// 2^22 bins: 513 us with one, 440 us so; L2 atomics: 210 G/s at best, 320 us; 2^25
+// into 256 bins 139 -> 90 us); 1 below 6 M, where few steps remain to overlap
+// (2^21 into 2^16 bins, the call: 29.3 us with four, 26.7; 1000 into 2^22, 22.6 and 20.7).
 // A bin's word only ever grows (max) or shrinks (min), so an element that does
 // not pass the word it reads needs no atomic: the k-th element of a bin passes
-// the earlier ones with probability 1/k.  Shared-memory words are always read
-// first; global ones when a bin has 64 elements or more on average (FILTER):
-// reading words that still change often makes copies of their lines on both
-// dies' sides of L2 (2^25 elements at 32 a bin 295 us with the read, 259
-// without; at 512 a bin, Zipf, 111 against 255).
+// the earlier ones with probability 1/k.  With V = 4, shared-memory words are
+// always read first; global ones when a bin has 256 elements or more on average
+// (FILTER): reading words that still change often makes copies of their lines on
+// both dies' sides of L2 (2^25 elements at 32 a bin 295 us with the read, 259
+// without; 2^23 at 128 a bin 81 and 76; 2^24 at 256 a bin 131 and 140; 2^25 at 512
+// a bin, Zipf, 111 and 255).
 template <class I, bool MAX, bool FILTER>
 __global__ void __launch_bounds__(kHistBlock, 3) hist_arg_f32_kernel(HistArgs A) {
     extern __shared__ unsigned char smem_raw[];
@@ -244,6 +247,42 @@ __global__ void __launch_bounds__(kHistBlock, 3) hist_arg_f32_kernel(HistArgs A)
             } else {
                 if (MAX) atomicMax(A.key + c[j], w[j]); else atomicMin(A.key + c[j], w[j]);
             }
+        }
+    }
+    __syncthreads();
+    for (int q = threadIdx.x; q < H; q += blockDim.x) {
+        const unsigned long long w = sh[q];
+        if (w != empty) {
+            if (MAX) atomicMax(A.key + q, w); else atomicMin(A.key + q, w);
+        }
+    }
+}
+
+// V = 1
+template <class I, bool MAX>
+__global__ void __launch_bounds__(kHistBlock, 4) hist_arg_f32_short_kernel(HistArgs A) {
+    extern __shared__ unsigned char smem_raw[];
+    unsigned long long* sh = reinterpret_cast<unsigned long long*>(smem_raw);
+    const unsigned long long empty = MAX ? 0ull : 0xffffffffffffffffull;
+    const int H = (int)std::min<int64_t>(A.m, kHistSmemKeys);
+    for (int b = threadIdx.x; b < H; b += blockDim.x) sh[b] = empty;
+    __syncthreads();
+    const I* inds = static_cast<const I*>(A.inds);
+    const float* vals = static_cast<const float*>(A.vals);
+    float* vb = static_cast<float*>(A.valsbar);
+    const bool fill = !A.accumulate && !A.primal_only;
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < A.n; i += stride) {
+        const int64_t c = ld_index(inds, i);
+        const float x = __ldcs(vals + i);
+        if (fill) __stcs(vb + i, 0.f);
+        if (c < 0 || c >= A.m) continue;
+        const unsigned long long w =
+            ((unsigned long long)orderkey_f32(x) << 32) | (MAX ? ~(uint32_t)i : (uint32_t)i);
+        if (c < H) {
+            if (MAX) atomicMax(sh + c, w); else atomicMin(sh + c, w);
+        } else {
+            if (MAX) atomicMax(A.key + c, w); else atomicMin(A.key + c, w);
         }
     }
     __syncthreads();
@@ -667,13 +706,15 @@ int run_hist(HistArgs A, cudaStream_t s) {
         const bool mx = op == ADPAR_OP_MAX;
         if constexpr (sizeof(T) == 4) {
             const size_t sh = (size_t)std::min<int64_t>(A.m, kHistSmemKeys) * 8;
-            const int g = (int)std::max<int64_t>(
-                1, std::min<int64_t>((A.n + 4 * kHistBlock - 1) / (4 * kHistBlock), (int64_t)sms * 3));
+            const bool one = A.n < kArgVector;
             const bool filter = A.n / kFilterPerBin >= A.m;
-            if (mx && filter) hist_arg_f32_kernel<I, true, true><<<g, kHistBlock, sh, s>>>(A);
-            else if (mx) hist_arg_f32_kernel<I, true, false><<<g, kHistBlock, sh, s>>>(A);
-            else if (filter) hist_arg_f32_kernel<I, false, true><<<g, kHistBlock, sh, s>>>(A);
-            else hist_arg_f32_kernel<I, false, false><<<g, kHistBlock, sh, s>>>(A);
+            const int V = one ? 1 : 4;
+            const int g = (int)std::max<int64_t>(
+                1, std::min<int64_t>((A.n + V * kHistBlock - 1) / (V * kHistBlock), (int64_t)sms * 3));
+            auto kernel = mx ? (filter ? hist_arg_f32_kernel<I, true, true> : hist_arg_f32_kernel<I, true, false>)
+                             : (filter ? hist_arg_f32_kernel<I, false, true> : hist_arg_f32_kernel<I, false, false>);
+            if (one) kernel = mx ? hist_arg_f32_short_kernel<I, true> : hist_arg_f32_short_kernel<I, false>;
+            kernel<<<g, kHistBlock, sh, s>>>(A);
         } else {
             if (mx) hist_arg_f64_key_kernel<I, true><<<gridN, kHistBlock, 0, s>>>(A);
             else hist_arg_f64_key_kernel<I, false><<<gridN, kHistBlock, 0, s>>>(A);
@@ -748,7 +789,8 @@ void configure_smem() {
         if constexpr (sizeof(I) == 8)
             cudaFuncSetAttribute(hist_logprod_kernel<I, I>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLogSmem);
         for (auto f : {hist_arg_f32_kernel<I, true, true>, hist_arg_f32_kernel<I, true, false>,
-                       hist_arg_f32_kernel<I, false, true>, hist_arg_f32_kernel<I, false, false>})
+                       hist_arg_f32_kernel<I, false, true>, hist_arg_f32_kernel<I, false, false>,
+                       hist_arg_f32_short_kernel<I, true>, hist_arg_f32_short_kernel<I, false>})
             cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024);
     }
 }
