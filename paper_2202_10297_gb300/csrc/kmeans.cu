@@ -368,7 +368,9 @@ __global__ void __launch_bounds__(KM_THREADS, 1)
             // the stage's tile (or the end marker), then the accumulator.  A
             // wait that gives up, or the end marker, makes the warp skip its
             // reads of the accumulator; the first barrier of the tile then
-            // takes every thread of the group out together
+            // takes both warps of the pair out together.  The other pairs and
+            // the MMA warp leave at the end marker of their own, or learn of a
+            // wait that gave up from s_abort, which every wait polls
             const bool okx = __all_sync(0xffffffffu, tc::mbar_wait(&x_full[s], (i / KM_STAGES) & 1, s_abort));
             const int64_t t = s_tile[s];
             const bool more = okx && t >= 0;
