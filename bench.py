@@ -524,7 +524,7 @@ def row_prod(args):
         t_log, t_val, t_pri = _cuda_ms(f_log, 200, 20), _cuda_ms(f_val, 200, 20), _cuda_ms(f_pri, 200, 20)
         cases["n65536_z%d" % z] = {"vjp_logdomain_us": 1e3 * t_log, "vjp_value_us": 1e3 * t_val,
                                    "primal_us": 1e3 * t_pri, "vjp_primal_ratio": t_val / t_pri,
-                                   "launches_per_call": 1,
+                                   "launches_value": 1, "launches_logdomain": 3,
                                    "oracle_elements_per_s": _oracle_rate(lambda: O.prod_reduce_vjp(a, 1.0), 65536, 1.0)}
     n = 1 << 28
     big = torch.rand(n, dtype=torch.float64, device="cuda") + 0.5
@@ -668,9 +668,9 @@ def row_jvp(args):
 
 # algorithmic bytes per element of the reduce_by_index VJPs: + reads the
 # indices and writes the adjoint (the bins' cotangents stay in L2); max also
-# reads the values in the recompute pass and the indices again in the
-# adjoint pass; * reads values and indices in both passes
-HIST_ALG_BYTES = {"add": 8, "max": 16, "mul": 20}
+# reads the values, in the one pass over the elements that it takes; * reads
+# values and indices in both passes
+HIST_ALG_BYTES = {"add": 8, "max": 12, "mul": 20}
 HIST_CASES = [(m, dist) for m in (256, 1 << 16, 1 << 22) for dist in ("uniform", "zipf")]
 
 
@@ -999,7 +999,7 @@ def default_rows(args):
     srv = row_serve(args)
     rows = {}
     c1 = {k: {kk: v[kk] for kk in ("vjp_value_us", "vjp_logdomain_us", "primal_us", "vjp_primal_ratio",
-                                   "launches_per_call", "oracle_elements_per_s")}
+                                   "launches_value", "launches_logdomain", "oracle_elements_per_s")}
           for k, v in prod["cases"].items() if k.startswith("n65536")}
     big = prod["cases"]["n2^28_f64_value"]
     c1["n2^28_f64"] = {"ms": big["ms"], "hbm_frac_of_measured": big["hbm_frac_of_measured"],
