@@ -468,8 +468,13 @@ size_t state_bytes(int op, int dtype) {
     return 0;
 }
 
-// resident blocks of the * kernels: 4 of 256 threads on each of 152 SMs
-constexpr int kProdGrid = 4 * 152;
+// resident blocks of the * kernels: 4 of 256 threads per SM
+int prod_wave() {
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    return std::min(4 * std::max(sms, 1), kRedMaxBlocks);
+}
 
 int grid_for(int64_t n, int dtype) {
     const int64_t per_block = (int64_t)kRedBlock * (dtype == ADPAR_F64 ? 2 : 4) * 8;
@@ -503,11 +508,12 @@ int run_reduce(ReduceArgs A, int op, cudaStream_t s) {
         }
         // one 16-byte vector per thread, up to a whole wave of resident blocks
         const int64_t per = (int64_t)kRedBlock * (16 / sizeof(T));
-        const int gp = (int)std::max<int64_t>(1, std::min<int64_t>((A.n + per - 1) / per, kProdGrid));
+        const int wave = prod_wave();
+        const int gp = (int)std::max<int64_t>(1, std::min<int64_t>((A.n + per - 1) / per, wave));
         reduce_prod_kernel<T><<<gp, kRedBlock, 0, s>>>(A);
         if (A.primal_only) break;
         // the log domain's threads form two FP64 logarithms of their own: four elements each
-        const int ga = A.logdomain ? (int)std::max<int64_t>(1, std::min<int64_t>((A.n + 1023) / 1024, kProdGrid)) : gp;
+        const int ga = A.logdomain ? (int)std::max<int64_t>(1, std::min<int64_t>((A.n + 1023) / 1024, wave)) : gp;
         prod_adjoint_kernel<T><<<ga, kRedBlock, 0, s>>>(A);
         break;
     }
