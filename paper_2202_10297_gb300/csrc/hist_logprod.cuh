@@ -160,6 +160,11 @@ __host__ __device__ inline void logprod_decode(ulonglong2 w, long long whole, un
 constexpr int kLogHot = 64;
 constexpr int kLogSlots = 8192;
 constexpr int kLogThreads = 1024;
+// Lanes of a warp up to which each adds both words of its bin in L2 itself: with
+// more, neighbouring lanes share the work, a request per bin.  2^25 elements, the
+// call, by neighbours always / so / each lane always: into 2^16 Zipf bins (3 such
+// lanes in a warp) 282 / 269 / 265 us; into 30000 uniform ones (23) 293 / 298 / 471.
+constexpr int kLogFew = 6;
 constexpr int kLogMaxSlots = 32 * kLogHot + kLogSlots;
 constexpr size_t kLogSmem = kLogTab * 16 + (size_t)kLogMaxSlots * 16;
 
@@ -196,8 +201,7 @@ __device__ __forceinline__ void ld_index4(const I* p, int64_t v, int64_t (&b)[4]
 // first is a multiple of 4); four consecutive elements per thread and step, the
 // next step's loaded while this one is added.  B: int, or int64_t for 2^31 bins
 // and more.  Bound by instruction issue: 2^25 elements into 2^16 Zipf bins take
-// 189 us (73% of the issue slots, the shared-memory pipe at 56%), into 256 bins
-// 143 us; reading the input alone takes 39, the compare-and-swap products that
+// 177 us (72% of the issue slots), into 256 bins 146 us (74%); reading the input alone takes 39, the compare-and-swap products that
 // were here took 1396 us, and terms in units of 2^-54 (a limb less) 174 us.
 template <class I, class B>
 __global__ void __launch_bounds__(kLogThreads, 1) hist_logprod_kernel(LogProdArgs A, int64_t first, int64_t last) {
@@ -269,21 +273,27 @@ __global__ void __launch_bounds__(kLogThreads, 1) hist_logprod_kernel(LogProdArg
                 if (add) atomicAdd(w2 + q, add);
                 bin = -1;
             }
-            if (__any_sync(0xffffffffu, bin >= 0)) {
-                // a bin's two words lie side by side: two neighbouring lanes add them
-                // in one request to its sector, the even lane's bin's first (a lane
-                // adding both words itself, 2^25 elements into 30000 bins: 470 us
-                // against 298)
-                const bool odd = lane & 1;
+            const unsigned far = __ballot_sync(0xffffffffu, bin >= 0);  // lanes whose bins are words in L2
+            if (far) {
                 const unsigned long long x = ((unsigned long long)(hi & 15u) << 32) | lo;
                 const unsigned long long y = (unsigned long long)(((long long)e << kLogHigh) + (long long)(hi >> 4)) +
                                              ((unsigned long long)neg << 32);
-                const unsigned long long other = __shfl_xor_sync(0xffffffffu, odd ? x : y, 1);
-                const B ob = __shfl_xor_sync(0xffffffffu, bin, 1);
-                const B b0 = odd ? ob : bin, b1 = odd ? bin : ob;
-                unsigned long long* w = reinterpret_cast<unsigned long long*>(A.acc) + odd;
-                if (b0 >= 0) red_add_u64(w + 2 * (int64_t)b0, odd ? other : x);
-                if (b1 >= 0) red_add_u64(w + 2 * (int64_t)b1, odd ? y : other);
+                unsigned long long* acc = reinterpret_cast<unsigned long long*>(A.acc);
+                if (__popc(far) <= kLogFew) {
+                    if (bin >= 0) {
+                        red_add_u64(acc + 2 * (int64_t)bin, x);
+                        red_add_u64(acc + 2 * (int64_t)bin + 1, y);
+                    }
+                } else {
+                    // a bin's two words lie side by side: two neighbouring lanes add them
+                    // in one request to its sector, the even lane's bin's first
+                    const bool odd = lane & 1;
+                    const unsigned long long other = __shfl_xor_sync(0xffffffffu, odd ? x : y, 1);
+                    const B ob = __shfl_xor_sync(0xffffffffu, bin, 1);
+                    const B b0 = odd ? ob : bin, b1 = odd ? bin : ob;
+                    if (b0 >= 0) red_add_u64(acc + 2 * (int64_t)b0 + odd, odd ? other : x);
+                    if (b1 >= 0) red_add_u64(acc + 2 * (int64_t)b1 + odd, odd ? y : other);
+                }
             }
         }
     }
