@@ -830,10 +830,11 @@ def row_scatter(args, inputs=None, map_acc=True):
         t = _cuda_ms(lambda: A.adpar_vjp_scatter(it, ysbar, vsbar=vsbar), 5, 2)
         # 16 B per j (is, the gathered ysbar, vsbar, the zeroed ysbar); a random
         # 4-byte access moves a 32-byte sector: 4 + 32 + 4 + 32 = 72 B per j
-        cases["sorted" if sort else "random"] = {
+        c = cases["sorted" if sort else "random"] = {
             "ms": t, "elements_per_s": m / t * 1e3, "gbs_algorithmic": 16 * m / t / 1e6,
-            "hbm_frac_of_measured": 16 * m / t / 1e6 / hbm, "gbs_sector": 72 * m / t / 1e6,
-            "sector_frac_of_measured": 72 * m / t / 1e6 / hbm}
+            "hbm_frac_of_measured": 16 * m / t / 1e6 / hbm}
+        if not sort:
+            c.update(gbs_sector=72 * m / t / 1e6, sector_frac_of_measured=72 * m / t / 1e6 / hbm)
         del it, ysbar, vsbar
     nj = 1 << 26
     for g, na, width in (("gather", 1 << 20, 1), ("scale", 1 << 20, 1), ("gather", 4096, 1),
@@ -1012,7 +1013,7 @@ def default_rows(args):
         "oracle": hist["cpu_baseline"]}
     rows["config3_scatter"] = {
         "n": 1 << 28, "m": 1 << 26, "bytes_per_element": 16,
-        "cases": {k: {kk: v[kk] for kk in ("ms", "hbm_frac_of_measured", "sector_frac_of_measured")}
+        "cases": {k: {kk: v[kk] for kk in ("ms", "hbm_frac_of_measured", "sector_frac_of_measured") if kk in v}
                   for k, v in sc["cases"].items()},
         "oracle": sc["cpu_baseline"]}
     rows["config4_batch"] = {k: batch[k] for k in ("segments", "elements", "graph_ms", "plain_calls_ms",

@@ -201,8 +201,9 @@ __device__ __forceinline__ void ld_index4(const I* p, int64_t v, int64_t (&b)[4]
 // first is a multiple of 4); four consecutive elements per thread and step, the
 // next step's loaded while this one is added.  B: int, or int64_t for 2^31 bins
 // and more.  Bound by instruction issue: 2^25 elements into 2^16 Zipf bins take
-// 177 us (72% of the issue slots), into 256 bins 146 us (74%); reading the input alone takes 39, the compare-and-swap products that
-// were here took 1396 us, and terms in units of 2^-54 (a limb less) 174 us.
+// 177 us (72% of the issue slots), into 256 bins 146 us (74%); reading the input
+// alone takes 39, the compare-and-swap products that were here took 1396 us, and
+// terms in units of 2^-54 (less closely held) 174 us.
 template <class I, class B>
 __global__ void __launch_bounds__(kLogThreads, 1) hist_logprod_kernel(LogProdArgs A, int64_t first, int64_t last) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
